@@ -8,6 +8,11 @@
 //   warp 1      TMEM allocator + MMA issuer: per 16-deep K step the 36 digit
 //               products with p + q < NS, product (p, q) into the group
 //               accumulator g = p + q (TMEM columns g * 64 .. g * 64 + 63).
+//               The digit planes of B are contiguous in a stage and so are the
+//               groups in TMEM, so digit p of A meets up to four digits of B
+//               in one MMA of N = 256: 12 MMAs instead of 36.  A 64-column MMA
+//               is bound by its operand reads from shared memory (6 KB for 32
+//               cycles of math); merged, a K step reads 120 KB instead of 216.
 //   warps 2..3  idle (registers come in groups of four warps)
 //   warps 4..11 epilogue (two warps per TMEM lane quarter, 32 columns each):
 //               every KCHUNK of K, the 8 group accumulators are folded in
@@ -40,7 +45,7 @@ constexpr int NTHREADS = 384;
 constexpr int EPI_WARP0 = 4;                                // warps 4..11: epilogue
 constexpr int EPI_THREADS = NTHREADS - 32 * EPI_WARP0;
 constexpr uint32_t TMEM_COLS = 512;
-constexpr uint32_t IDESC = tc::idesc_f32acc(1u /*BF16*/, BM, BN);
+constexpr int QMERGE = 4;  // digits of B per MMA (N = 256, the widest)
 constexpr int CHUNK_STAGES = KCHUNK / BK;
 static_assert(NS * BN <= (int)TMEM_COLS, "group accumulators must fit in TMEM");
 
@@ -60,15 +65,15 @@ static_assert(sizeof(Shared) <= BAR_BYTES, "barrier block");
 // hi 2^-31 + lo 2^-63 (lo unsigned, below 2^32).  Each G_g is an integer held
 // exactly in FP32 (below 2^24, see the header), so the chunk's sum is formed
 // in integer arithmetic: groups 2..7 by Horner in 64 bits, T = sum_{g>=2}
-// G_g 2^(7(7-g)), |T| < 2^59 (|G_g| < 2^23.4 for g >= 1 with KCHUNK = 256:
+// G_g 2^(7(7-g)), |T| < 2^59 (|G_g| < 2^24 for g >= 1 with KCHUNK = 384:
 // at most two products of a leading digit, |d_0| <= 128, and g - 1 of
 // trailing digits, |d_p| <= 64, per K term), and groups 0..1 as Q = 2^7 G_0
-// + G_1, |Q| < 2^30 (|G_0| <= 2^22).  The chunk's value is Q 2^-21 + T 2^-63
+// + G_1, |Q| < 2^30 (|G_0| <= 384 * 2^14, |G_1| <= 384 * 2^14).  The chunk's value is Q 2^-21 + T 2^-63
 // = (2^10 Q + floor(T / 2^32)) 2^-31 + (T mod 2^32) 2^-63; the low word's
 // carry moves into hi, which grows by less than 2^41 per chunk.  No FP64
 // instruction runs per chunk: the FP64 pipe, GB300's slowest unit, is used
 // once per output at the end of the item (fixed_to_double).
-static_assert(NS == 8 && SLICE_BITS == 7 && KCHUNK <= 256, "fold_groups is written for 8 digits of 7 bits");
+static_assert(NS == 8 && SLICE_BITS == 7 && KCHUNK <= 384, "fold_groups is written for 8 digits of 7 bits");
 __device__ __forceinline__ void fold_groups(const uint32_t (&r)[NS][2], int x, long long &hi, unsigned &lo) {
   int gi[NS];
 #pragma unroll
@@ -96,6 +101,30 @@ __device__ inline void raise_timeout(Shared *sh, int *status) {
 // 2^e for integer e in the normal range (exact).
 __device__ inline double exp2i(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 __device__ inline int exp_of(const int *exps, long i) { return max(exps[i] - kExpBias, kExpMin); }
+// x 2^e for any int e (exact up to the ends of the FP64 range); NaN where e
+// carries the poison of a row with an infinity or a NaN.
+__device__ inline double scale2(double x, int e) {
+  if (abs(e) <= 1000) return x * exp2i(e);
+  if (e > kExpPoison / 2) return __longlong_as_double(0x7ff8000000000000ll);
+  const int e1 = max(-1000, min(1000, e));
+  return x * exp2i(e1) * exp2i(max(-1000, min(1000, e - e1)));
+}
+// x 2^-e for the exponent e of x's row: |x 2^-e| < 1; 0 in a poisoned row.
+__device__ inline double unit_scaled(double x, int e) { return e > kExpPoison / 2 ? 0.0 : scale2(x, -e); }
+// Biased exponent of a row whose largest magnitude is m (> 0); bad: it holds
+// an infinity or a NaN.
+__device__ inline int biased_exp(double m, bool bad) {
+  if (bad) return kExpPoison;
+  int e;
+  frexp(m, &e);  // m = f 2^e, f in [0.5, 1): every |x| < 2^e
+  return e + kExpBias;
+}
+// |x|, or +infinity for a NaN (fmax would drop it)
+__device__ inline double mag(double x) {
+  const double a = fabs(x);
+  return a <= 1.7976931348623157e308 ? a : __longlong_as_double(0x7ff0000000000000ll);
+}
+__device__ inline bool is_inf(double m) { return m > 1.7976931348623157e308; }
 
 // The NS digits of v (|v| < 1) written d[0], d[plane], ...: v is rounded to
 // X = v 2^56 (an integer below 2^56; the unit of the last digit is 2^-56),
@@ -131,17 +160,13 @@ __global__ void __launch_bounds__(256)
   for (int c = blockIdx.z * 8 + w; c < nb; c += 8 * gridDim.z) {
     size_t o = base + r + (size_t)c * nb;
     double x = f64 ? t64[o] : (double)t32[o];
-    m = fmax(m, fabs(x));
+    m = fmax(m, mag(x));
   }
   red[w][lane] = m;
   __syncthreads();
   if (w == 0) {
     for (int q = 1; q < 8; q++) m = fmax(m, red[q][lane]);
-    if (m > 0.0) {
-      int e;
-      frexp(m, &e);  // m = f 2^e, f in [0.5, 1): every |x| < 2^e
-      atomicMax(&exps[jb.z + r], e + kExpBias);
-    }
+    if (m > 0.0) atomicMax(&exps[jb.z + r], biased_exp(m, is_inf(m)));
   }
 }
 
@@ -170,7 +195,7 @@ __global__ void __launch_bounds__(256)
   for (int q = 0; q < 4; q++) {
     int rr = w + 8 * q;
     int r = r0 + rr;
-    double v = blk[rr][lane] * exp2i(-exp_of(exps, (long)jb.z + r));  // exact: |v| < 1
+    double v = unit_scaled(blk[rr][lane], exp_of(exps, (long)jb.z + r));  // exact: |v| < 1
     write_digits(v, digits + (size_t)jb.y * NS * plane + (size_t)r * nb + c0 + lane, plane);
   }
 }
@@ -188,16 +213,12 @@ __global__ void __launch_bounds__(256)
   const int r = blockIdx.x * 32 + lane;
   double m = 0.0;
   if (r < nrows)
-    for (long c = (long)blockIdx.y * 8 + w; c < ncols; c += 8L * gridDim.y) m = fmax(m, fabs(X[r + (col0 + c) * ld]));
+    for (long c = (long)blockIdx.y * 8 + w; c < ncols; c += 8L * gridDim.y) m = fmax(m, mag(X[r + (col0 + c) * ld]));
   red[w][lane] = m;
   __syncthreads();
   if (w == 0 && r < nrows) {
     for (int q = 1; q < 8; q++) m = fmax(m, red[q][lane]);
-    if (m > 0.0) {
-      int e;
-      frexp(m, &e);
-      atomicMax(&exps[r], e + kExpBias);
-    }
+    if (m > 0.0) atomicMax(&exps[r], biased_exp(m, is_inf(m)));
   }
 }
 
@@ -221,7 +242,7 @@ __global__ void __launch_bounds__(256)
   const size_t plane = (size_t)npad * kpad;
   for (int q = 0; q < 4; q++) {
     const int rr = w + 8 * q, r = r0 + rr;
-    const double v = blk[rr][lane] * exp2i(-exp_of(exps, r));  // exact: |v| < 1
+    const double v = unit_scaled(blk[rr][lane], exp_of(exps, r));  // exact: |v| < 1
     write_digits(v, digits + (size_t)r * kpad + c0 + lane, plane);
   }
 }
@@ -239,22 +260,21 @@ __global__ void __launch_bounds__(256)
   const double *z = Z + blk.x + (size_t)c * ldz;
   double m = 0.0;
   if (c < s)
-    for (int r = threadIdx.x; r < blk.y; r += blockDim.x) m = fmax(m, fabs(z[r]));
+    for (int r = threadIdx.x; r < blk.y; r += blockDim.x) m = fmax(m, mag(z[r]));
   for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int q = 1; q < (int)(blockDim.x >> 5); q++) m = fmax(m, red[q]);
-    int e = 0;
-    if (m > 0.0) frexp(m, &e);
-    s_e = e;
-    exps[(long)b * s_pad + c] = e + kExpBias;
+    const int eb = m > 0.0 ? biased_exp(m, is_inf(m)) : kExpBias;
+    s_e = max(eb - kExpBias, kExpMin);
+    exps[(long)b * s_pad + c] = eb;
   }
   __syncthreads();
-  const double inv = exp2i(-s_e);
+  const int e = s_e;
   size_t plane = (size_t)s_pad * zcols;
   for (int r = threadIdx.x; r < blk.y; r += blockDim.x)
-    write_digits((c < s) ? z[r] * inv : 0.0, digits + (size_t)c * zcols + blk.x + r, plane);
+    write_digits((c < s) ? unit_scaled(z[r], e) : 0.0, digits + (size_t)c * zcols + blk.x + r, plane);
 }
 
 // ------------------------------------------------------- blocked TRSM
@@ -269,15 +289,14 @@ __device__ inline void row_digits_tw(const double (&x)[NQ], int *e_out, uint16_t
   const int lane = threadIdx.x & 31;
   double m = 0.0;
 #pragma unroll
-  for (int q = 0; q < NQ; q++) m = fmax(m, fabs(x[q]));
+  for (int q = 0; q < NQ; q++) m = fmax(m, mag(x[q]));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-  int e = 0;
-  if (m > 0.0) frexp(m, &e);  // every |x| < 2^e
-  if (lane == 0) *e_out = (m > 0.0) ? e + kExpBias : 0;
-  const double sc = exp2i(-((m > 0.0) ? max(e, kExpMin) : kExpMin));  // exact: |x sc| < 1
+  const int eb = m > 0.0 ? biased_exp(m, is_inf(m)) : 0;
+  if (lane == 0) *e_out = eb;
+  const int e = max(eb - kExpBias, kExpMin);
 #pragma unroll
-  for (int q = 0; q < NQ; q++) write_digits(x[q] * sc, d + 32 * q + lane, plane);
+  for (int q = 0; q < NQ; q++) write_digits(unit_scaled(x[q], e), d + 32 * q + lane, plane);  // exact: below 1
 }
 
 // Digits of L_kk's column blocks: one CTA per (32 rows, block J), warp w
@@ -461,13 +480,15 @@ __global__ void __maxnreg__(168)
 #pragma unroll
             for (int p = 0; p < NS; p++) {
               const uint64_t ad = tc::desc_add(a0, p * A_SL + ks * 32);
+              // digits q .. q + nq - 1 of B: groups p + q .. p + q + nq - 1
 #pragma unroll
-              for (int q = 0; q < NS - p; q++) {
-                const int g = p + q;
+              for (int q = 0; q < NS - p; q += QMERGE) {
+                const int nq = NS - p - q < QMERGE ? NS - p - q : QMERGE;
                 const uint64_t bd = tc::desc_add(b0, q * B_SL + ks * 32);
-                tc::mma_f16(tmem + (uint32_t)(g * BN), ad, bd, IDESC, (started >> g) & 1u);
-                started |= 1u << g;
+                tc::mma_f16(tmem + (uint32_t)((p + q) * BN), ad, bd, tc::idesc_f32acc(1u /*BF16*/, BM, nq * BN),
+                            p > 0 ? 1u : started);
               }
+              started = 1u;  // digit 0 of A has written every group
             }
           }
           tc::mma_commit(&sh->empty[stage]);
@@ -543,7 +564,7 @@ __global__ void __maxnreg__(168)
 #pragma unroll
           for (int x = 0; x < 8; x++) {
             const int cx = col0 + x0 + x;
-            double v = fixed_to_double(hi[x0 + x], lo[x0 + x]) * exp2i(ea + exp_of(b_exp, (long)item.b_sc + cx));
+            double v = scale2(fixed_to_double(hi[x0 + x], lo[x0 + x]), ea + exp_of(b_exp, (long)item.b_sc + cx));
             if (MODE == TC64_SUB)
               __stcg(o + (long)cx * ldo, cv[x] - v);
             else if (cx < item.cols_valid)

@@ -28,7 +28,10 @@ constexpr int BK = 32;         // K per pipeline stage
 constexpr int STAGES = 2;
 constexpr int NS = 8;          // digits per operand entry
 constexpr int SLICE_BITS = 7;
-constexpr int KCHUNK = 256;    // K accumulated exactly in FP32 between FP64 flushes
+// K accumulated exactly in FP32 between two drains of the group accumulators:
+// |sum| <= 384 (2 * 128 * 64 + 6 * 64^2) = 15,728,640 < 2^24 (leading digits
+// |d_0| <= 128, the others <= 64).  256 drained 1.5 times as often.
+constexpr int KCHUNK = 384;
 
 // One BM x BN output block: the sum over its segments of A_seg B_seg^T.
 // Operand row r of digit plane p sits at arena row (row + p * plane); every
@@ -53,9 +56,11 @@ emu_status make_map(emu_ctx *ctx, CUtensorMap *map, const void *base, uint64_t i
 
 // Exponent arrays hold e + kExpBias, so that a zeroed array (cudaMemset 0)
 // holds the lowest exponent; readers clamp e at kExpMin, which only rows of
-// zeros reach.
+// zeros reach.  A row with an infinity or a NaN holds kExpPoison: its digits
+// are zeros and every product with it is NaN, as in floating point.
 constexpr int kExpBias = 1024;
 constexpr int kExpMin = -960;
+constexpr int kExpPoison = 1 << 20;
 
 // Row exponents of listed tiles: jobs {tile, -, exponent base}; a tile is read
 // from the FP64 arena when its class is FP64, else from the FP32 master.  Row
