@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "emu_internal.h"
+#include "factor64.h"
 #include "gemm_f64.h"
 #include "mixed.h"
 
@@ -600,8 +601,9 @@ static emu_status collect_status(emu_ctx *ctx, int *pivot) {
   return EMU_OK;
 }
 
-// Plain FP64 right-looking tile Cholesky: POTRF(k), TRSM(:,k), SYRK/GEMM of
-// the trailing tiles, k = 0 .. NT-1.
+// Plain FP64 right-looking tile Cholesky on the FP64 pipe, for the tile sizes
+// the digit form does not take: POTRF(k), TRSM(:,k), SYRK/GEMM of the trailing
+// tiles, k = 0 .. NT-1.
 static emu_status factor64(emu_ctx *ctx, emu_mat *A) {
   for (int k = 0; k < A->nt; k++) {
     emu_status s = launch_potrf64_tile(ctx, A, k);
@@ -629,7 +631,8 @@ extern "C" emu_status emu_potrf_mp(emu_ctx *ctx, emu_mat *A, const emu_mp_opts *
   } else if (mixed) {
     s = factor_mixed(ctx, A, o);
   } else {
-    s = factor64(ctx, A);
+    s = factor64_digits_supports(A) ? factor64_digits(ctx, A) : EMU_ENOMEM;
+    if (s == EMU_ENOMEM) s = factor64(ctx, A);
   }
   if (s != EMU_OK) return s;
   EMU_CUDA_TRY(ctx, cudaEventRecord(ctx->ev1, ctx->stream));
@@ -677,8 +680,10 @@ extern "C" emu_status emu_sample(emu_ctx *ctx, const emu_mat *L, int nsamples, u
   if (s == EMU_OK) {
     if (L->cs)
       s = classfmt_sample(ctx, L, Z, npad, nsamples, dY, ldy);
-    else if (L->state == MAT_FACTOR64)
-      s = launch_trmm64(ctx, L, Z, npad, nsamples, dY, ldy);
+    else if (L->state == MAT_FACTOR64) {
+      s = factor64_digits_supports(L) ? sample64_digits(ctx, L, Z, npad, nsamples, dY, ldy) : EMU_ENOMEM;
+      if (s == EMU_ENOMEM) s = launch_trmm64(ctx, L, Z, npad, nsamples, dY, ldy);
+    }
     else
       s = mixed_sample(ctx, L, Z, npad, nsamples, dY, ldy);
   }

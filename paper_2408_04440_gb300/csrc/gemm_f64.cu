@@ -14,10 +14,12 @@
 //               is bound by its operand reads from shared memory (6 KB for 32
 //               cycles of math); merged, a K step reads 120 KB instead of 216.
 //   warps 2..3  idle (registers come in groups of four warps)
-//   warps 4..11 epilogue (two warps per TMEM lane quarter, 32 columns each):
+//   warps 4..19 epilogue (four warps per TMEM lane quarter, 16 columns each;
+//               eight warps of 32 columns left the schedulers idle between
+//               dependent integer steps):
 //               every KCHUNK of K, the 8 group accumulators are folded in
 //               integer arithmetic into exact fixed-point accumulators
-//               (fold_groups), converted to FP64 once per item;
+//               (fold_groups), rounded to FP64 once per item (fixed_scaled);
 //               after the last chunk the row scales are applied and the block
 //               is subtracted from the FP64 output.
 // The 8 accumulators fill TMEM, so the MMA warp waits for the epilogue to
@@ -39,10 +41,9 @@ constexpr int STAGE_BYTES = NS * (A_SL + B_SL);       // 96 KB
 constexpr int RING_BYTES = STAGES * STAGE_BYTES;
 constexpr int BAR_BYTES = 128;
 constexpr int SMEM_BYTES = RING_BYTES + BAR_BYTES + 1024;  // + alignment slack
-// 12 warps: registers are granted per group of four warps, so a 10-warp
-// CTA would be charged for 12 at the same per-thread count.
-constexpr int NTHREADS = 384;
-constexpr int EPI_WARP0 = 4;                                // warps 4..11: epilogue
+constexpr int NTHREADS = 640;
+constexpr int EPI_WARP0 = 4;                                // warps 4..19: epilogue
+constexpr int EC = 16;                                      // output columns per epilogue thread
 constexpr int EPI_THREADS = NTHREADS - 32 * EPI_WARP0;
 constexpr uint32_t TMEM_COLS = 512;
 constexpr int QMERGE = 4;  // digits of B per MMA (N = 256, the widest)
@@ -71,8 +72,8 @@ static_assert(sizeof(Shared) <= BAR_BYTES, "barrier block");
 // + G_1, |Q| < 2^30 (|G_0| <= 384 * 2^14, |G_1| <= 384 * 2^14).  The chunk's value is Q 2^-21 + T 2^-63
 // = (2^10 Q + floor(T / 2^32)) 2^-31 + (T mod 2^32) 2^-63; the low word's
 // carry moves into hi, which grows by less than 2^41 per chunk.  No FP64
-// instruction runs per chunk: the FP64 pipe, GB300's slowest unit, is used
-// once per output at the end of the item (fixed_to_double).
+// instruction runs per chunk: the FP64 pipe, GB300's slowest unit, is used for
+// one add per output at the end of the item.
 static_assert(NS == 8 && SLICE_BITS == 7 && KCHUNK <= 384, "fold_groups is written for 8 digits of 7 bits");
 __device__ __forceinline__ void fold_groups(const uint32_t (&r)[NS][2], int x, long long &hi, unsigned &lo) {
   int gi[NS];
@@ -86,8 +87,42 @@ __device__ __forceinline__ void fold_groups(const uint32_t (&r)[NS][2], int x, l
   hi += q * 1024 + (t >> 32) + (l < lo ? 1 : 0);  // arithmetic shift: floor; carry of the low word
   lo = l;
 }
-__device__ __forceinline__ double fixed_to_double(long long hi, unsigned lo) {
-  return fma((double)hi, 0x1p-31, (double)lo * 0x1p-63);
+// (hi 2^-31 + lo 2^-63) 2^s rounded once to FP64 (ties to even), for s that
+// keeps the result in the normal range: normalised, rounded and packed in
+// integer arithmetic.  Two conversions, an FMA and a multiply on the FP64 pipe
+// took about 20 k cycles per 128 x 64 block, as long as the MMAs of K = 256.
+// s out of range: the same value through FP64 arithmetic (fixed_scaled_any).
+__device__ double fixed_scaled_any(long long hi, unsigned lo, int s);
+__device__ __forceinline__ double fixed_scaled(long long hi, unsigned lo, int s) {
+  const bool neg = hi < 0;
+  // |hi 2^32 + lo| = ahi 2^32 + alo
+  const unsigned alo = neg ? 0u - lo : lo;
+  const unsigned long long ahi = (unsigned long long)(neg ? ~hi + (lo == 0u) : hi);
+  unsigned long long t;  // the leading 64 bits, top bit set
+  int lz;
+  bool sticky = false;
+  if (ahi != 0) {
+    lz = __clzll((long long)ahi);
+    t = ahi << lz;
+    if (lz >= 32) {
+      t |= (unsigned long long)alo << (lz - 32);
+    } else {
+      t |= (unsigned long long)alo >> (32 - lz);
+      sticky = (alo << lz) != 0u;
+    }
+  } else {
+    if (alo == 0u) return s > kExpPoison / 2 ? fixed_scaled_any(hi, lo, s) : 0.0;  // a poisoned row's digits are 0
+    const int l = __clz((int)alo);
+    t = (unsigned long long)alo << (32 + l);
+    lz = 64 + l;
+  }
+  const int e = 1055 - lz + s;  // biased exponent
+  if (e < 1 || e > 2045) return fixed_scaled_any(hi, lo, s);
+  unsigned long long m = t >> 11;
+  const unsigned rem = (unsigned)t & 0x7ffu;
+  m += (rem > 0x400u || (rem == 0x400u && (sticky || (m & 1ull)))) ? 1ull : 0ull;
+  m += (unsigned long long)(e - 1) << 52;  // the implicit bit adds one to the exponent; so does a carry
+  return __longlong_as_double((long long)(m | (neg ? 0x8000000000000000ull : 0ull)));
 }
 
 __device__ inline bool failed(const int *st) { return *((volatile const int *)st) != DEV_OK; }
@@ -101,44 +136,88 @@ __device__ inline void raise_timeout(Shared *sh, int *status) {
 // 2^e for integer e in the normal range (exact).
 __device__ inline double exp2i(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 __device__ inline int exp_of(const int *exps, long i) { return max(exps[i] - kExpBias, kExpMin); }
-// x 2^e for any int e (exact up to the ends of the FP64 range); NaN where e
+// fixed_scaled for any s: near the ends of the FP64 range, and NaN where s
 // carries the poison of a row with an infinity or a NaN.
-__device__ inline double scale2(double x, int e) {
-  if (abs(e) <= 1000) return x * exp2i(e);
-  if (e > kExpPoison / 2) return __longlong_as_double(0x7ff8000000000000ll);
-  const int e1 = max(-1000, min(1000, e));
-  return x * exp2i(e1) * exp2i(max(-1000, min(1000, e - e1)));
+__device__ __noinline__ double fixed_scaled_any(long long hi, unsigned lo, int s) {
+  if (s > kExpPoison / 2) return __longlong_as_double(0x7ff8000000000000ll);
+  const double x = fma((double)hi, 0x1p-31, (double)lo * 0x1p-63);
+  const int s1 = max(-1000, min(1000, s));
+  return x * exp2i(s1) * exp2i(max(-1000, min(1000, s - s1)));
 }
-// x 2^-e for the exponent e of x's row: |x 2^-e| < 1; 0 in a poisoned row.
-__device__ inline double unit_scaled(double x, int e) { return e > kExpPoison / 2 ? 0.0 : scale2(x, -e); }
-// Biased exponent of a row whose largest magnitude is m (> 0); bad: it holds
-// an infinity or a NaN.
-__device__ inline int biased_exp(double m, bool bad) {
-  if (bad) return kExpPoison;
-  int e;
-  frexp(m, &e);  // m = f 2^e, f in [0.5, 1): every |x| < 2^e
-  return e + kExpBias;
+// Magnitude bits of x: ordered like |x|, infinities and then NaNs on top, so
+// that row maxima are taken in integers.
+__device__ inline unsigned long long mag_bits(double x) {
+  return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
 }
-// |x|, or +infinity for a NaN (fmax would drop it)
-__device__ inline double mag(double x) {
-  const double a = fabs(x);
-  return a <= 1.7976931348623157e308 ? a : __longlong_as_double(0x7ff0000000000000ll);
+// Biased exponent of a row whose largest magnitude bits are m > 0: every
+// |x| < 2^(result - kExpBias).  (The sign is masked again: the compiler takes
+// the mask above for an FP64 absolute value, which may keep a NaN's sign.)
+__device__ inline int biased_exp(unsigned long long m) {
+  const int ex = (int)(m >> 52) & 0x7ff;
+  if (ex == 0x7ff) return kExpPoison;
+  return (ex > 0 ? ex - 1022 : (64 - __clzll((long long)m)) - 1074) + kExpBias;
 }
-__device__ inline bool is_inf(double m) { return m > 1.7976931348623157e308; }
+// x 2^(56 - e) rounded to the nearest integer (ties to even), for |x| < 2^e:
+// below 2^56 in magnitude.  In integer arithmetic on the significand: the FP64
+// pipe issues about one warp instruction per 19 cycles and SM, and a multiply
+// and a conversion per entry there took longer than the entry's memory traffic.
+// 0 where e is a poisoned row's.
+__device__ inline long long to_fixed(double x, int e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  int ex = (int)(b >> 52) & 0x7ff;
+  unsigned long long m = b & 0xfffffffffffffull;
+  if (ex > 0) m |= 1ull << 52;
+  else ex = 1;
+  const int sh = ex - 1019 - e;  // x 2^(56 - e) = m 2^sh, sh <= 3
+  unsigned long long X;
+  if (sh >= 0) {
+    X = m << sh;
+  } else {
+    const int r = -sh < 54 ? -sh : 54;  // m < 2^53: 2^-54 m rounds to 0
+    X = (m + ((1ull << (r - 1)) - 1) + ((m >> r) & 1ull)) >> r;
+  }
+  return (long long)b < 0 ? -(long long)X : (long long)X;
+}
 
-// The NS digits of v (|v| < 1) written d[0], d[plane], ...: v is rounded to
-// X = v 2^56 (an integer below 2^56; the unit of the last digit is 2^-56),
-// then the digits are peeled off from the top in integer arithmetic, each
-// rounded to nearest, so |digit 0| <= 128 and |digit p| <= 64 for p >= 1 and
-// sum_p digit_p 2^(7 (NS - 1 - p)) = X exactly.
-__device__ inline void write_digits(double v, uint16_t *d, size_t plane) {
-  long long X = __double2ll_rn(v * 0x1p56);
+// The NS digits of X (|X| <= 2^56, the unit of the last digit is 2^-56): peeled
+// off from the top, each rounded to nearest, so |digit 0| <= 128 and
+// |digit p| <= 64 for p >= 1 and sum_p digit_p 2^(7 (NS - 1 - p)) = X exactly.
+// As BF16 bits: a digit is at most eight bits wide, so the upper half of its
+// FP32 pattern (formed by an add of 1.5 2^23, no conversion) is exact.
+__device__ inline void digit_bits(long long X, uint32_t (&d)[NS]) {
 #pragma unroll
   for (int p = 0; p < NS; p++) {
     const int sh = SLICE_BITS * (NS - 1 - p);
-    long long dg = (sh > 0) ? ((X + (1LL << (sh > 0 ? sh - 1 : 0))) >> sh) : X;
+    const long long dg = (sh > 0) ? ((X + (1LL << (sh > 0 ? sh - 1 : 0))) >> sh) : X;
     X -= dg << sh;
-    d[p * plane] = __bfloat16_as_ushort(__float2bfloat16_rn((float)(int)dg));  // small integer: exact
+    d[p] = __float_as_uint(__int_as_float(0x4B400000 + (int)dg) - 12582912.0f) >> 16;
+  }
+}
+// Digits of v with row exponent e written d[0], d[plane], ...
+__device__ inline void write_digits(double v, int e, uint16_t *d, size_t plane) {
+  uint32_t g[NS];
+  digit_bits(to_fixed(v, e), g);
+#pragma unroll
+  for (int p = 0; p < NS; p++) d[p * plane] = (uint16_t)g[p];
+}
+// The same for two neighbouring columns (d 4-byte aligned).
+__device__ inline void write_digits2(double v0, double v1, int e, uint16_t *d, size_t plane) {
+  uint32_t g0[NS], g1[NS];
+  digit_bits(to_fixed(v0, e), g0);
+  digit_bits(to_fixed(v1, e), g1);
+#pragma unroll
+  for (int p = 0; p < NS; p++) *reinterpret_cast<uint32_t *>(d + p * plane) = g0[p] | (g1[p] << 16);
+}
+// A 32 x 32 block (256 threads) in shared memory, row rr with exponent
+// exp(rr), to its digit planes at d + rr * ld: a half warp per row, two
+// columns per lane.
+template <class Exp>
+__device__ inline void write_block_digits(const double (&blk)[32][33], Exp exp, uint16_t *d, size_t ld, size_t plane) {
+  const int h = threadIdx.x >> 4, c = 2 * (threadIdx.x & 15);
+#pragma unroll
+  for (int q = 0; q < 2; q++) {
+    const int rr = h + 16 * q;
+    write_digits2(blk[rr][c], blk[rr][c + 1], exp(rr), d + (size_t)rr * ld + c, plane);
   }
 }
 
@@ -150,23 +229,23 @@ __global__ void __launch_bounds__(256)
     k_rowexp64(const double *__restrict__ t64, const float *__restrict__ t32, const unsigned char *__restrict__ cls,
                const int4 *__restrict__ jobs, int nb, int *__restrict__ exps, const int *st) {
   if (failed(st)) return;
-  __shared__ double red[8][33];
+  __shared__ unsigned long long red[8][33];
   int4 jb = jobs[blockIdx.y];
   size_t base = (size_t)jb.x * nb * nb;
   bool f64 = cls[jb.x] == EMU_CLASS_FP64;
   int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int r = blockIdx.x * 32 + lane;
-  double m = 0.0;
+  unsigned long long m = 0;
   for (int c = blockIdx.z * 8 + w; c < nb; c += 8 * gridDim.z) {
     size_t o = base + r + (size_t)c * nb;
     double x = f64 ? t64[o] : (double)t32[o];
-    m = fmax(m, mag(x));
+    m = max(m, mag_bits(x));
   }
   red[w][lane] = m;
   __syncthreads();
   if (w == 0) {
-    for (int q = 1; q < 8; q++) m = fmax(m, red[q][lane]);
-    if (m > 0.0) atomicMax(&exps[jb.z + r], biased_exp(m, is_inf(m)));
+    for (int q = 1; q < 8; q++) m = max(m, red[q][lane]);
+    if (m > 0) atomicMax(&exps[jb.z + r], biased_exp(m));
   }
 }
 
@@ -192,12 +271,8 @@ __global__ void __launch_bounds__(256)
   }
   __syncthreads();
   size_t plane = (size_t)nb * nb;
-  for (int q = 0; q < 4; q++) {
-    int rr = w + 8 * q;
-    int r = r0 + rr;
-    double v = unit_scaled(blk[rr][lane], exp_of(exps, (long)jb.z + r));  // exact: |v| < 1
-    write_digits(v, digits + (size_t)jb.y * NS * plane + (size_t)r * nb + c0 + lane, plane);
-  }
+  write_block_digits(blk, [&](int rr) { return exp_of(exps, (long)jb.z + r0 + rr); },
+                     digits + (size_t)jb.y * NS * plane + (size_t)r0 * nb + c0, nb, plane);
 }
 
 // Row exponents of a dense column-major block X[0:nrows, col0:col0+ncols]
@@ -208,17 +283,17 @@ __global__ void __launch_bounds__(256)
     k_rowexp_dense(const double *__restrict__ X, long ld, int nrows, long col0, long ncols, int *__restrict__ exps,
                    const int *st) {
   if (failed(st)) return;
-  __shared__ double red[8][33];
+  __shared__ unsigned long long red[8][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int r = blockIdx.x * 32 + lane;
-  double m = 0.0;
+  unsigned long long m = 0;
   if (r < nrows)
-    for (long c = (long)blockIdx.y * 8 + w; c < ncols; c += 8L * gridDim.y) m = fmax(m, mag(X[r + (col0 + c) * ld]));
+    for (long c = (long)blockIdx.y * 8 + w; c < ncols; c += 8L * gridDim.y) m = max(m, mag_bits(X[r + (col0 + c) * ld]));
   red[w][lane] = m;
   __syncthreads();
   if (w == 0 && r < nrows) {
-    for (int q = 1; q < 8; q++) m = fmax(m, red[q][lane]);
-    if (m > 0.0) atomicMax(&exps[r], biased_exp(m, is_inf(m)));
+    for (int q = 1; q < 8; q++) m = max(m, red[q][lane]);
+    if (m > 0) atomicMax(&exps[r], biased_exp(m));
   }
 }
 
@@ -239,34 +314,30 @@ __global__ void __launch_bounds__(256)
     blk[lane][cc] = (r < nrows && c < ncols) ? X[r + (col0 + c) * ld] : 0.0;
   }
   __syncthreads();
-  const size_t plane = (size_t)npad * kpad;
-  for (int q = 0; q < 4; q++) {
-    const int rr = w + 8 * q, r = r0 + rr;
-    const double v = unit_scaled(blk[rr][lane], exp_of(exps, r));  // exact: |v| < 1
-    write_digits(v, digits + (size_t)r * kpad + c0 + lane, plane);
-  }
+  write_block_digits(blk, [&](int rr) { return exp_of(exps, r0 + rr); }, digits + (size_t)r0 * kpad + c0, kpad,
+                     (size_t)npad * kpad);
 }
 
 // Digits of Z columns per matrix block: one CTA per (sample c < s_pad, block).
 // The exponent covers the block's rows of column c; samples c >= s are zero.
 __global__ void __launch_bounds__(256)
     k_slicez64(const double *__restrict__ Z, long ldz, int s, int s_pad, const int2 *__restrict__ blocks, long zcols,
-               int *__restrict__ exps, uint16_t *__restrict__ digits, const int *st) {
+               int2 whole, int *__restrict__ exps, uint16_t *__restrict__ digits, const int *st) {
   if (failed(st)) return;
-  __shared__ double red[8];
+  __shared__ unsigned long long red[8];
   __shared__ int s_e;
   int c = blockIdx.x, b = blockIdx.y;
-  int2 blk = blocks[b];
+  int2 blk = blocks ? blocks[b] : whole;
   const double *z = Z + blk.x + (size_t)c * ldz;
-  double m = 0.0;
+  unsigned long long m = 0;
   if (c < s)
-    for (int r = threadIdx.x; r < blk.y; r += blockDim.x) m = fmax(m, mag(z[r]));
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
+    for (int r = threadIdx.x; r < blk.y; r += blockDim.x) m = max(m, mag_bits(z[r]));
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_down_sync(0xffffffffu, m, o));
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int q = 1; q < (int)(blockDim.x >> 5); q++) m = fmax(m, red[q]);
-    const int eb = m > 0.0 ? biased_exp(m, is_inf(m)) : kExpBias;
+    for (int q = 1; q < (int)(blockDim.x >> 5); q++) m = max(m, red[q]);
+    const int eb = m > 0 ? biased_exp(m) : kExpBias;
     s_e = max(eb - kExpBias, kExpMin);
     exps[(long)b * s_pad + c] = eb;
   }
@@ -274,7 +345,7 @@ __global__ void __launch_bounds__(256)
   const int e = s_e;
   size_t plane = (size_t)s_pad * zcols;
   for (int r = threadIdx.x; r < blk.y; r += blockDim.x)
-    write_digits((c < s) ? unit_scaled(z[r], e) : 0.0, digits + (size_t)c * zcols + blk.x + r, plane);
+    write_digits((c < s) ? z[r] : 0.0, e, digits + (size_t)c * zcols + blk.x + r, plane);
 }
 
 // ------------------------------------------------------- blocked TRSM
@@ -287,16 +358,16 @@ static_assert(TW % 32 == 0 && TW % BN == 0, "block width");
 // at d[c + p plane].
 __device__ inline void row_digits_tw(const double (&x)[NQ], int *e_out, uint16_t *d, size_t plane) {
   const int lane = threadIdx.x & 31;
-  double m = 0.0;
+  unsigned long long m = 0;
 #pragma unroll
-  for (int q = 0; q < NQ; q++) m = fmax(m, mag(x[q]));
+  for (int q = 0; q < NQ; q++) m = max(m, mag_bits(x[q]));
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-  const int eb = m > 0.0 ? biased_exp(m, is_inf(m)) : 0;
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  const int eb = m > 0 ? biased_exp(m) : 0;
   if (lane == 0) *e_out = eb;
   const int e = max(eb - kExpBias, kExpMin);
 #pragma unroll
-  for (int q = 0; q < NQ; q++) write_digits(unit_scaled(x[q], e), d + 32 * q + lane, plane);  // exact: below 1
+  for (int q = 0; q < NQ; q++) write_digits(x[q], e, d + 32 * q + lane, plane);
 }
 
 // Digits of L_kk's column blocks: one CTA per (32 rows, block J), warp w
@@ -368,13 +439,169 @@ __global__ void __launch_bounds__(128)
   }
 }
 
+// Digits of whole rows of a packed FP64 matrix (launch_panel_digits): one CTA
+// per PR rows, over the tile columns [tcol0, tcol0 + tcols) (tcols < 0: up to
+// the row's tile): the rows' maxima in one pass, then the digits in a second
+// one whose reads hit L2.  One launch where a memset, a maximum pass over all
+// tiles and a slicing pass took three.
+constexpr int PR = 32;
+__global__ void __launch_bounds__(256)
+    k_panel_digits(const double *__restrict__ t64, int NT, int nb, int row0, int tcol0, int tcols, int e_row0,
+                   int *__restrict__ exps, int d_row0, long plane, long kpad, uint16_t *__restrict__ digits,
+                   const int *st) {
+  if (failed(st)) return;
+  __shared__ double blk[32][33];
+  __shared__ unsigned long long red[8][33];
+  __shared__ int se[32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int r0 = row0 + blockIdx.x * PR, ti = r0 / nb, rin = r0 % nb;
+  const int t1 = tcols < 0 ? ti + 1 : tcol0 + tcols;
+  const size_t te = (size_t)nb * nb;
+  unsigned long long m = 0;
+  for (int tj = tcol0; tj < t1; tj++) {
+    const double *T = t64 + (size_t)tile_index(ti, tj, NT) * te + rin + lane;
+#pragma unroll 4
+    for (int c = w; c < nb; c += 8) m = max(m, mag_bits(T[(size_t)c * nb]));
+  }
+  red[w][lane] = m;
+  __syncthreads();
+  if (w == 0) {
+    for (int q = 1; q < 8; q++) m = max(m, red[q][lane]);
+    const int eb = m > 0 ? biased_exp(m) : 0;
+    exps[r0 + lane - e_row0] = eb;
+    se[lane] = max(eb - kExpBias, kExpMin);
+  }
+  for (int tj = tcol0; tj < t1; tj++) {
+    const double *T = t64 + (size_t)tile_index(ti, tj, NT) * te + rin + lane;
+    for (int c0 = 0; c0 < nb; c0 += 32) {
+      double v[4];
+#pragma unroll
+      for (int q = 0; q < 4; q++) v[q] = T[(size_t)(c0 + w + 8 * q) * nb];
+      __syncthreads();
+#pragma unroll
+      for (int q = 0; q < 4; q++) blk[lane][w + 8 * q] = v[q];
+      __syncthreads();
+      write_block_digits(blk, [&](int rr) { return se[rr]; },
+                         digits + (size_t)(r0 - d_row0) * kpad + (long)(tj - tcol0) * nb + c0, kpad,
+                         (size_t)plane * kpad);
+    }
+  }
+}
+
+// The same for one tile column and nb <= kPanelCols: eight rows per CTA, read
+// once into shared memory (32-row CTAs of the two-pass kernel took 27 us for
+// one 512-wide tile, 16 CTAs).
+constexpr int kPanelCols = 2048, P8 = 8;
+__global__ void __launch_bounds__(256)
+    k_panel_digits8(const double *__restrict__ t64, int NT, int nb, int row0, int tj, int *__restrict__ exps,
+                    long plane, uint16_t *__restrict__ digits, const int *st) {
+  if (failed(st)) return;
+  extern __shared__ double pv[];  // [8][nb + 2]
+  __shared__ unsigned long long red[8][P8 + 1];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, ld = nb + 2;
+  const int r0 = row0 + blockIdx.x * P8, ti = r0 / nb, rin = r0 % nb;
+  // a warp reads four columns of the eight rows (64 bytes each) at a time
+  const int rr = lane & 7, cc = w * 4 + (lane >> 3);
+  const double *T = t64 + (size_t)tile_index(ti, tj, NT) * nb * nb + rin + rr;
+  unsigned long long m = 0;
+#pragma unroll 8
+  for (int c = cc; c < nb; c += 32) {
+    const double x = T[(size_t)c * nb];
+    m = max(m, mag_bits(x));
+    pv[rr * ld + c] = x;
+  }
+#pragma unroll
+  for (int o = 8; o < 32; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane < P8) red[w][lane] = m;
+  __syncthreads();
+  // warp w: row w
+  unsigned long long mr = red[lane & 7][w];
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) mr = max(mr, __shfl_xor_sync(0xffffffffu, mr, o));
+  const int eb = mr > 0 ? biased_exp(mr) : 0, e = max(eb - kExpBias, kExpMin);
+  if (lane == 0) exps[r0 + w] = eb;
+  uint16_t *d = digits + (size_t)(r0 + w) * nb;
+  for (int c = 2 * lane; c < nb; c += 64) write_digits2(pv[w * ld + c], pv[w * ld + c + 1], e, d + c, (size_t)plane * nb);
+}
+
 // ------------------------------------------------------------- GEMM
-template <int MODE>
-__global__ void __maxnreg__(168)
+// Items of a region in groups of RG_W column blocks: in a group the row
+// blocks run in order and each meets the group's columns, so that the items
+// in flight on the chip share their operands' rows in L2 (152 CTAs cover about
+// 19 row blocks by 8 column blocks).
+constexpr int RG_W = 8;
+struct Work {
+  long out_off;
+  int a_sc, b_sc, rows_valid, cols_valid;
+  int a_row, b_row;
+  int total;  // K stages (0: nothing to do)
+};
+// First row block of column group g.
+template <int SRC>
+__host__ __device__ inline int group_row0(const Region &rg, int g) {
+  if (SRC != SRC_SYRK) return rg.r_lo;
+  const int d = (rg.c_lo + g * RG_W) * BN / BM;  // the diagonal's row block
+  return d > rg.r_lo ? d : rg.r_lo;
+}
+template <int SRC>
+__host__ __device__ inline int group_items(const Region &rg, int g) {
+  const int c = rg.c_lo + g * RG_W, w = rg.c_hi - c < RG_W ? rg.c_hi - c : RG_W;
+  const int h = rg.r_hi - group_row0<SRC>(rg, g);
+  return h > 0 ? w * h : 0;
+}
+template <int SRC>
+__host__ __device__ inline int region_items(const Region &rg) {
+  int n = 0;
+  for (int g = 0; rg.c_lo + g * RG_W < rg.c_hi; g++) n += group_items<SRC>(rg, g);
+  return n;
+}
+struct Cursor {  // the group of the last item found; items come in ascending order
+  int g = 0, base = 0;
+};
+template <int SRC>
+__device__ inline Work region_work(const Region &rg, Cursor &cur, int it, long ldo) {
+  int cnt;
+  while (it >= cur.base + (cnt = group_items<SRC>(rg, cur.g))) {
+    cur.base += cnt;
+    cur.g++;
+  }
+  const int q = it - cur.base, c0 = rg.c_lo + cur.g * RG_W, wd = min(RG_W, rg.c_hi - c0);
+  const int R = group_row0<SRC>(rg, cur.g) + q / wd, C = c0 + q % wd;
+  const int row = R * BM, col = C * BN, nb = rg.nb;
+  Work w;
+  w.rows_valid = BM;
+  w.cols_valid = BN;
+  w.total = nb / BK;
+  if (SRC == SRC_SYRK) {
+    if (row + BM - 1 < col) w.total = 0;  // above the diagonal
+    w.out_off = tile_index(row / nb, col / nb, rg.NT) * (long)nb * nb + row % nb + (long)(col % nb) * nb;
+    w.a_row = w.a_sc = row;
+    w.b_row = w.b_sc = col;
+  } else if (SRC == SRC_TRSM) {
+    const int z = row / nb, rin = row % nb, slot = rg.slot0 + z;
+    w.total = TW / BK;
+    w.out_off = (long)rg.tiles[z] * nb * nb + rin + (long)col * nb;
+    w.a_row = slot * NS * nb + rin;
+    w.a_sc = slot * nb + rin;
+    w.b_row = rg.J * NS * nb + col;
+    w.b_sc = rg.J * nb + col;
+  } else {
+    w.total = (row / nb + 1) * nb / BK;
+    w.out_off = row + (long)col * ldo;
+    w.a_row = w.a_sc = row - rg.a_row0;
+    w.b_row = w.b_sc = col;
+    w.rows_valid = min(BM, rg.rows_valid - row);
+    w.cols_valid = min(BN, rg.cols_valid - col);
+  }
+  return w;
+}
+
+template <int MODE, int SRC>
+__global__ void __maxnreg__(96)
     k_tc_gemm64(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap,
                 const Item *__restrict__ items, int nitems, const Seg *__restrict__ segs, int nb, int a_plane,
                 int b_plane, const int *__restrict__ a_exp, const int *__restrict__ b_exp,
-                double *__restrict__ out, int ldo, int *status) {
+                double *__restrict__ out, long ldo, int *status, const Region rg) {
   extern __shared__ uint8_t smem_raw[];
   uint32_t raw_addr = tc::smem_u32(smem_raw);
   uint32_t pad = ((raw_addr + 1023u) & ~1023u) - raw_addr;
@@ -414,11 +641,23 @@ __global__ void __maxnreg__(168)
       int stage = 0;
       uint32_t phase = 0;
       bool ok = *abort == 0;
+      Cursor cur;
       for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x) {
-        Item item = items[it];
-        for (int sg = item.seg_begin; sg < item.seg_end && ok; sg++) {
-          Seg sd = segs[sg];
-          for (int kc = 0; kc < kstages; kc++) {
+        int sg0 = 0, sg1 = 1, kst = kstages;
+        Seg sd;
+        if constexpr (SRC == SRC_LIST) {
+          sg0 = items[it].seg_begin;
+          sg1 = items[it].seg_end;
+        } else {
+          const Work wk = region_work<SRC>(rg, cur, it, ldo);
+          kst = wk.total;
+          sd.a_row = wk.a_row;
+          sd.b_row = wk.b_row;
+          sd.a_x = sd.b_x = 0;
+        }
+        for (int sg = sg0; sg < sg1 && ok; sg++) {
+          if constexpr (SRC == SRC_LIST) sd = segs[sg];
+          for (int kc = 0; kc < kst; kc++) {
             if (!tc::mbar_wait(&sh->empty[stage], phase ^ 1u, abort)) {
               raise_timeout(sh, status);
               ok = false;
@@ -452,9 +691,13 @@ __global__ void __maxnreg__(168)
       uint32_t chunk = 0;
       uint32_t started = 0;
       bool ok = *abort == 0;
+      Cursor cur;
       for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x) {
-        Item item = items[it];
-        const int total = (item.seg_end - item.seg_begin) * kstages;  // K stages of the item
+        int total;  // K stages of the item
+        if constexpr (SRC == SRC_LIST)
+          total = (items[it].seg_end - items[it].seg_begin) * kstages;
+        else
+          total = region_work<SRC>(rg, cur, it, ldo).total;
         for (int ks_i = 0; ks_i < total && ok; ks_i++) {
           if (ks_i % CHUNK_STAGES == 0) {
             // the epilogue has read the previous chunk's accumulators
@@ -507,23 +750,43 @@ __global__ void __maxnreg__(168)
     }
   } else if (warp >= EPI_WARP0) {
     // ------------------------------------------------------------ epilogue
-    // warps 4..11: TMEM lane quarter warp % 4 (the lanes a warp may access),
-    // columns [half * 32, half * 32 + 32) of the block
+    // TMEM lane quarter warp % 4 (the lanes a warp may access), columns
+    // [col0, col0 + EC) of the block
     const int quarter = warp & 3;
-    const int half = (warp - EPI_WARP0) >> 2;
     const int row = quarter * 32 + lane;
-    const int col0 = half * 32;
+    const int col0 = ((warp - EPI_WARP0) >> 2) * EC;
     const uint32_t tlane = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)col0;
     uint32_t chunk = 0;
     bool ok = *abort == 0;
+    Cursor cur;
     for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x) {
-      Item item = items[it];
-      const int total = (item.seg_end - item.seg_begin) * kstages;
+      Work item;
+      if constexpr (SRC == SRC_LIST) {
+        const Item li = items[it];
+        item.out_off = li.out_off;
+        item.a_sc = li.a_sc;
+        item.b_sc = li.b_sc;
+        item.rows_valid = li.rows_valid;
+        item.cols_valid = li.cols_valid;
+        item.total = (li.seg_end - li.seg_begin) * kstages;
+      } else {
+        item = region_work<SRC>(rg, cur, it, ldo);
+        if (item.total == 0) continue;  // every role skips it
+      }
+      const int total = item.total;
       const int nchunks = (total + CHUNK_STAGES - 1) / CHUNK_STAGES;
-      long long hi[32];
-      unsigned lo[32];
+      constexpr bool kWhole = MODE == TC64_SUB;  // every row and column exists
+      double *o = out + item.out_off + row;
+      if constexpr (kWhole) {
+        // the warp's 32 rows x EC columns (two 128-byte lines per column) on
+        // their way to L2 while the MMAs run
+        const double *pf = o - lane + (long)(col0 + (lane >> 1)) * ldo + (lane & 1) * 16;
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(pf));
+      }
+      long long hi[EC];
+      unsigned lo[EC];
 #pragma unroll
-      for (int x = 0; x < 32; x++) {
+      for (int x = 0; x < EC; x++) {
         hi[x] = 0;
         lo[x] = 0u;
       }
@@ -535,7 +798,7 @@ __global__ void __maxnreg__(168)
         }
         tc::fence_after_sync();
 #pragma unroll
-        for (int h = 0; h < 16; h++) {
+        for (int h = 0; h < EC / 2; h++) {
           uint32_t r[NS][2];
 #pragma unroll
           for (int g = 0; g < NS; g++) tc::tmem_ld_32x32b_x2(tlane + (uint32_t)(g * BN + h * 2), r[g]);
@@ -550,25 +813,27 @@ __global__ void __maxnreg__(168)
       if (!ok) break;
       // scales 2^(e_row + e_col), exact; then the output block
       const int ea = exp_of(a_exp, (long)item.a_sc + row);
-      double *o = out + item.out_off + row;
       // in groups of 8 columns: 8 loads in flight, then 8 stores
-      if (MODE == TC64_SUB || row < item.rows_valid) {
+      if (kWhole || row < item.rows_valid) {
 #pragma unroll
-        for (int x0 = 0; x0 < 32; x0 += 8) {
+        for (int x0 = 0; x0 < EC; x0 += 8) {
           double cv[8];
 #pragma unroll
           for (int x = 0; x < 8; x++) {
             const int cx = col0 + x0 + x;
-            cv[x] = (MODE == TC64_SUB || cx < item.cols_valid) ? __ldcg(o + (long)cx * ldo) : 0.0;
+            if constexpr (MODE == TC64_SET)
+              cv[x] = 0.0;
+            else
+              cv[x] = (kWhole || cx < item.cols_valid) ? __ldcg(o + (long)cx * ldo) : 0.0;
           }
 #pragma unroll
           for (int x = 0; x < 8; x++) {
             const int cx = col0 + x0 + x;
-            double v = scale2(fixed_to_double(hi[x0 + x], lo[x0 + x]), ea + exp_of(b_exp, (long)item.b_sc + cx));
+            double v = fixed_scaled(hi[x0 + x], lo[x0 + x], ea + exp_of(b_exp, (long)item.b_sc + cx));
             if (MODE == TC64_SUB)
               __stcg(o + (long)cx * ldo, cv[x] - v);
-            else if (cx < item.cols_valid)
-              __stcg(o + (long)cx * ldo, cv[x] + v);
+            else if (kWhole || cx < item.cols_valid)
+              __stcg(o + (long)cx * ldo, MODE == TC64_SET ? v : cv[x] + v);
           }
         }
       }
@@ -613,8 +878,18 @@ emu_status launch_slice_z(emu_ctx *ctx, const double *Z, long ldz, int s, int s_
                           int nblocks, long zcols, int *exps, uint16_t *digits) {
   if (nblocks <= 0 || s_pad <= 0) return EMU_OK;
   ProfScope ps(ctx, PROF_SPLIT, 0.0, (8.0 + 2.0 * NS) * (double)s_pad * zcols);
-  k_slicez64<<<dim3(s_pad, nblocks), 256, 0, ctx->stream>>>(Z, ldz, s, s_pad, d_blocks, zcols, exps, digits,
-                                                            ctx->d_status);
+  k_slicez64<<<dim3(s_pad, nblocks), 256, 0, ctx->stream>>>(Z, ldz, s, s_pad, d_blocks, zcols, int2{0, 0}, exps,
+                                                            digits, ctx->d_status);
+  EMU_LAUNCHED(ctx);
+  return EMU_OK;
+}
+
+emu_status launch_slice_cols(emu_ctx *ctx, const double *Z, long ldz, int s, int s_pad, int rows, int *exps,
+                             uint16_t *digits) {
+  if (s_pad <= 0 || rows <= 0) return EMU_OK;
+  ProfScope ps(ctx, PROF_SPLIT, 0.0, (8.0 + 2.0 * NS) * (double)s_pad * rows);
+  k_slicez64<<<s_pad, 256, 0, ctx->stream>>>(Z, ldz, s, s_pad, nullptr, rows, int2{0, rows}, exps, digits,
+                                             ctx->d_status);
   EMU_LAUNCHED(ctx);
   return EMU_OK;
 }
@@ -654,23 +929,120 @@ emu_status launch_trsm_block(emu_ctx *ctx, double *t64, int nb, const int *d_til
   return EMU_OK;
 }
 
+template <int MODE, int SRC>
+static emu_status launch_kernel(emu_ctx *ctx, int grid, const CUtensorMap &a, const CUtensorMap &b,
+                                const Item *d_items, int nitems, const Seg *d_segs, int nb, int a_plane, int b_plane,
+                                const int *a_exp, const int *b_exp, double *out, long ldo, const Region &rg) {
+  static std::atomic<uint64_t> attr{0};
+  EMU_CUDA_TRY(ctx, smem_limit_once(attr, ctx->device, (const void *)k_tc_gemm64<MODE, SRC>, SMEM_BYTES));
+  k_tc_gemm64<MODE, SRC><<<grid, NTHREADS, SMEM_BYTES, ctx->stream>>>(a, b, d_items, nitems, d_segs, nb, a_plane,
+                                                                      b_plane, a_exp, b_exp, out, ldo,
+                                                                      ctx->d_status, rg);
+  EMU_LAUNCHED(ctx);
+  return EMU_OK;
+}
+
 emu_status launch(emu_ctx *ctx, const CUtensorMap &a, const CUtensorMap &b, const Item *d_items, int nitems,
                   const Seg *d_segs, int nb, int a_plane, int b_plane, const int *a_exp, const int *b_exp, int mode,
                   double *out64, int ldo, int max_ctas) {
   if (nitems <= 0) return EMU_OK;
   if (nb % BK != 0) return EMU_EINVAL;
-  static std::atomic<uint64_t> attr_sub{0}, attr_add{0};
-  EMU_CUDA_TRY(ctx, smem_limit_once(attr_sub, ctx->device, (const void *)k_tc_gemm64<TC64_SUB>, SMEM_BYTES));
-  EMU_CUDA_TRY(ctx, smem_limit_once(attr_add, ctx->device, (const void *)k_tc_gemm64<TC64_ADD>, SMEM_BYTES));
   int grid = nitems < max_ctas ? nitems : max_ctas;
-  if (mode == TC64_SUB)
-    k_tc_gemm64<TC64_SUB><<<grid, NTHREADS, SMEM_BYTES, ctx->stream>>>(a, b, d_items, nitems, d_segs, nb, a_plane,
-                                                                       b_plane, a_exp, b_exp, out64, ldo,
-                                                                       ctx->d_status);
-  else
-    k_tc_gemm64<TC64_ADD><<<grid, NTHREADS, SMEM_BYTES, ctx->stream>>>(a, b, d_items, nitems, d_segs, nb, a_plane,
-                                                                       b_plane, a_exp, b_exp, out64, ldo,
-                                                                       ctx->d_status);
+  return mode == TC64_SUB ? launch_kernel<TC64_SUB, SRC_LIST>(ctx, grid, a, b, d_items, nitems, d_segs, nb, a_plane,
+                                                              b_plane, a_exp, b_exp, out64, ldo, Region())
+                          : launch_kernel<TC64_ADD, SRC_LIST>(ctx, grid, a, b, d_items, nitems, d_segs, nb, a_plane,
+                                                              b_plane, a_exp, b_exp, out64, ldo, Region());
+}
+
+emu_status launch_region(emu_ctx *ctx, int src, const CUtensorMap &a, const CUtensorMap &b, const Region &rg,
+                         int a_plane, int b_plane, const int *a_exp, const int *b_exp, double *out, long ldo,
+                         int max_ctas) {
+  if (rg.nb % BM != 0) return EMU_EINVAL;
+  const int n = src == SRC_SYRK ? region_items<SRC_SYRK>(rg) : region_items<SRC_TRMM>(rg);
+  if (n <= 0) return EMU_OK;
+  const int grid = std::max(1, std::min(n, max_ctas));
+#define EMU_REGION(M, S) \
+  launch_kernel<M, S>(ctx, grid, a, b, nullptr, n, nullptr, rg.nb, a_plane, b_plane, a_exp, b_exp, out, ldo, rg)
+  if (src == SRC_SYRK) return EMU_REGION(TC64_SUB, SRC_SYRK);
+  if (src == SRC_TRSM) return EMU_REGION(TC64_SUB, SRC_TRSM);
+  return EMU_REGION(TC64_SET, SRC_TRMM);
+#undef EMU_REGION
+}
+
+// Parts of a TrsmPlan, in order; off[i] is part i's start, the last entry the size.
+static void trsm_plan_parts(int nb, int slots, size_t (&off)[7]) {
+  const size_t nJ = nb / TW, plane = (size_t)nb * TW;
+  const size_t bytes[6] = {slots * nb * sizeof(int),
+                           slots * NS * plane * sizeof(uint16_t),
+                           nJ * nb * sizeof(int),
+                           std::max<size_t>(nJ - 1, 1) * NS * plane * sizeof(uint16_t),
+                           (size_t)nb * 32 * sizeof(double),
+                           (size_t)nb * sizeof(double)};
+  off[0] = 0;
+  for (int i = 0; i < 6; i++) off[i + 1] = off[i] + ((bytes[i] + 255) & ~(size_t)255);
+}
+size_t trsm_plan_bytes(int nb, int slots) {
+  size_t off[7];
+  trsm_plan_parts(nb, slots, off);
+  return off[6];
+}
+emu_status trsm_plan_init(emu_ctx *ctx, TrsmPlan *P, char *base, int nb, int slots) {
+  if (nb % TW != 0 || nb % BM != 0) return EMU_EINVAL;
+  size_t off[7];
+  trsm_plan_parts(nb, slots, off);
+  P->xexp = reinterpret_cast<int *>(base + off[0]);
+  P->xdig = reinterpret_cast<uint16_t *>(base + off[1]);
+  P->lexp = reinterpret_cast<int *>(base + off[2]);
+  P->ldig = reinterpret_cast<uint16_t *>(base + off[3]);
+  P->ls = reinterpret_cast<double *>(base + off[4]);
+  P->rinv = reinterpret_cast<double *>(base + off[5]);
+  emu_status s = make_map(ctx, &P->mx, P->xdig, TW, (uint64_t)slots * NS * nb, BM);
+  return s == EMU_OK ? make_map(ctx, &P->ml, P->ldig, TW, std::max<uint64_t>(nb / TW - 1, 1) * NS * nb, BN) : s;
+}
+emu_status trsm_plan_prep(emu_ctx *ctx, const TrsmPlan &P, const double *Lkk, int nb) {
+  emu_status s = launch_trsm64_prep(ctx, Lkk, nb, P.ls, P.rinv);
+  return s == EMU_OK ? launch_lkk_digits(ctx, Lkk, nb, P.lexp, P.ldig) : s;
+}
+emu_status trsm_plan_solve(emu_ctx *ctx, const TrsmPlan &P, double *t64, int nb, const int *d_tiles, int n,
+                           const double *Lkk, int slot0) {
+  if (n <= 0) return EMU_OK;
+  const int nJ = nb / TW;
+  Region rg;
+  rg.nb = nb;
+  rg.r_hi = n * (nb / BM);
+  rg.tiles = d_tiles;
+  rg.slot0 = slot0;
+  for (int J = 0; J < nJ; J++) {
+    const bool last = J + 1 == nJ;
+    emu_status s = launch_trsm_block(ctx, t64, nb, d_tiles, n, Lkk, J, P.ls, P.rinv, slot0, P.xexp,
+                                     last ? nullptr : P.xdig);
+    if (s != EMU_OK || last) return s;
+    rg.J = J;
+    rg.c_lo = (J + 1) * (TW / BN);
+    rg.c_hi = nb / BN;
+    if ((s = launch_region(ctx, SRC_TRSM, P.mx, P.ml, rg, nb, nb, P.xexp, P.lexp, t64, nb, ctx->sm_count)) != EMU_OK)
+      return s;
+  }
+  return EMU_OK;
+}
+
+emu_status launch_panel_digits(emu_ctx *ctx, const double *t64, int NT, int nb, int row0, int nrows, int tcol0,
+                               int tcols, int e_row0, int *exps, int d_row0, long plane, long kpad,
+                               uint16_t *digits) {
+  if (nb % PR != 0 || row0 % PR != 0 || nrows % PR != 0 || kpad % 2 != 0) return EMU_EINVAL;
+  if (nrows <= 0) return EMU_OK;
+  ProfScope ps(ctx, PROF_SPLIT, 0.0, (8.0 + 2.0 * NS) * nrows * (double)kpad);
+  if (tcols == 1 && nb <= kPanelCols && e_row0 == 0 && d_row0 == 0 && kpad == nb) {
+    static std::atomic<uint64_t> attr{0};
+    const int sm = P8 * (nb + 2) * (int)sizeof(double);
+    EMU_CUDA_TRY(ctx, smem_limit_once(attr, ctx->device, (const void *)k_panel_digits8,
+                                      P8 * (kPanelCols + 2) * (int)sizeof(double)));
+    k_panel_digits8<<<nrows / P8, 256, sm, ctx->stream>>>(t64, NT, nb, row0, tcol0, exps, plane, digits, ctx->d_status);
+    EMU_LAUNCHED(ctx);
+    return EMU_OK;
+  }
+  k_panel_digits<<<nrows / PR, 256, 0, ctx->stream>>>(t64, NT, nb, row0, tcol0, tcols, e_row0, exps, d_row0, plane,
+                                                      kpad, digits, ctx->d_status);
   EMU_LAUNCHED(ctx);
   return EMU_OK;
 }

@@ -48,7 +48,8 @@ struct Item {
   int seg_begin, seg_end;      // segments [seg_begin, seg_end)
   int rows_valid, cols_valid;  // rows / columns of the block that exist (TC64_ADD)
 };
-enum { TC64_SUB = 0, TC64_ADD = 1 };  // out -= A B^T (factor) / out += A B^T (samples, bounded)
+// out -= A B^T (factor) / out += A B^T / out = A B^T (the last two bounded by rows_valid, cols_valid)
+enum { TC64_SUB = 0, TC64_ADD = 1, TC64_SET = 2 };
 
 // 2-D BF16 tensor map over a digit arena of `inner` columns, box rows x 32.
 emu_status make_map(emu_ctx *ctx, CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows,
@@ -78,6 +79,10 @@ emu_status launch_slice(emu_ctx *ctx, const double *t64, const float *t32, const
 emu_status launch_slice_z(emu_ctx *ctx, const double *Z, long ldz, int s, int s_pad, const int2 *d_blocks,
                           int nblocks, long zcols, int *exps, uint16_t *digits);
 
+// The same for one block of all `rows` rows (no block list).
+emu_status launch_slice_cols(emu_ctx *ctx, const double *Z, long ldz, int s, int s_pad, int rows, int *exps,
+                             uint16_t *digits);
+
 // Row exponents and digit planes of a dense column-major FP64 block
 // X[0:nrows, col0:col0+ncols] (leading dimension ld): exps[r] for r < npad
 // (zeroed first), plane p of row r at digits + (p * npad + r) * kpad, K-major,
@@ -103,6 +108,60 @@ emu_status launch_lkk_digits(emu_ctx *ctx, const double *Lkk, int nb, int *exps,
 // exps[s nb + r], plane p of row r at arena row (s NS + p) nb + r (TW columns).
 emu_status launch_trsm_block(emu_ctx *ctx, double *t64, int nb, const int *d_tiles, int ntiles, const double *Lkk,
                              int J, const double *Ls, const double *rinvs, int slot0, int *exps, uint16_t *digits);
+
+// Implicit item sets: the items of one step of the plain FP64 factor, of the
+// blocked FP64-class TRSM and of the sampler, found from the item number by
+// every role of the kernel, so that no item lists are built, copied or read
+// (n = 160000 would need 5 GB of them).  Rows are counted in blocks of BM,
+// columns in blocks of BN (nb a multiple of BM).
+struct Region {
+  int NT = 0, nb = 0;
+  int J = 0;                 // column block of L_kk (TRSM)
+  int r_lo = 0, r_hi = 0;    // row blocks [r_lo, r_hi) (of the padded matrix; TRSM: of the listed tiles)
+  int c_lo = 0, c_hi = 0;    // column blocks [c_lo, c_hi) (of the padded matrix; TRSM: of the tile)
+  const int *tiles = nullptr;  // TRSM: tile indices; tile z has slot slot0 + z
+  int slot0 = 0;
+  int a_row0 = 0;            // TRMM: matrix row held by arena row 0 of A
+  int rows_valid = 0, cols_valid = 0;  // TRMM: rows / columns of the output that exist
+};
+// SYRK: out = t64: tiles (r, c) -= A_r B_c^T for the blocks of the region on
+//   or below the diagonal; A and B rows are matrix rows of a panel's digits.
+// TRSM: out = t64: column block c of the listed tiles -= X_J L_cJ^T; X digits
+//   per slot (launch_trsm_block), L_kk digits of block J (launch_lkk_digits).
+// TRMM: out(row, col) = A_row B_col^T over K = the row's tiles 0 .. row / nb,
+//   out column-major; A rows start at matrix row a_row0.
+enum { SRC_LIST = 0, SRC_SYRK = 1, SRC_TRSM = 2, SRC_TRMM = 3 };
+emu_status launch_region(emu_ctx *ctx, int src, const CUtensorMap &a, const CUtensorMap &b, const Region &rg,
+                         int a_plane, int b_plane, const int *a_exp, const int *b_exp, double *out, long ldo,
+                         int max_ctas);
+
+// Row exponents and digits of rows [row0, row0 + nrows) of the tile columns
+// [col0, ncols) (in tiles; ncols < 0: up to the row's own tile) of a packed
+// FP64 matrix: exps[r - e_row0], plane p of row r at arena row
+// p * plane + r - d_row0, K-major with kpad columns.  One exponent per row.
+// Tiles above the diagonal are not read.  row0, nrows multiples of 32.
+emu_status launch_panel_digits(emu_ctx *ctx, const double *t64, int NT, int nb, int row0, int nrows, int tcol0,
+                               int tcols, int e_row0, int *exps, int d_row0, long plane, long kpad,
+                               uint16_t *digits);
+
+// Workspace of the blocked FP64-class TRSM over `slots` tiles of size nb.
+struct TrsmPlan {
+  int *xexp = nullptr;
+  uint16_t *xdig = nullptr;   // solved blocks: slot s, plane p, row r at (s NS + p) nb + r, TW columns
+  int *lexp = nullptr;        // L_kk's column blocks (launch_lkk_digits)
+  uint16_t *ldig = nullptr;
+  double *ls = nullptr, *rinv = nullptr;  // launch_trsm64_prep
+  CUtensorMap mx, ml;
+};
+size_t trsm_plan_bytes(int nb, int slots);
+// Lays the plan out in `base` (trsm_plan_bytes, 256-byte aligned) and encodes its maps.
+emu_status trsm_plan_init(emu_ctx *ctx, TrsmPlan *P, char *base, int nb, int slots);
+// Per panel, after its POTRF: the pre-scaled diagonal blocks and the digits of
+// L_kk's column blocks.
+emu_status trsm_plan_prep(emu_ctx *ctx, const TrsmPlan &P, const double *Lkk, int nb);
+// X = A L_kk^{-T} in place for the tiles d_tiles[0 .. n) (slots slot0 ..).
+emu_status trsm_plan_solve(emu_ctx *ctx, const TrsmPlan &P, double *t64, int nb, const int *d_tiles, int n,
+                           const double *Lkk, int slot0);
 
 // out64 (-= or +=) per item, K = nb per segment, on at most max_ctas persistent
 // CTAs; a_plane / b_plane = arena rows between digit planes.
