@@ -18,6 +18,7 @@
 
 #include "emu_internal.h"
 #include "rng.cuh"
+#include "sht_digits.h"
 
 namespace {
 
@@ -342,28 +343,19 @@ __global__ void __launch_bounds__(128) k_emulate_grid(const double *__restrict__
 }  // namespace
 
 
-extern "C" {
+// A transform runs as digit products from this bandlimit or this much work on.
+// Its dozen launches take 105 us (inverse) and 170 us (forward) however small
+// it is; measured against the direct sums on ntheta = 1.5 L, nphi = 2.5 L
+// (inverse / forward, us): L = 24, 100 steps (2.5e7, 3.7e7 flops) 111 against
+// 115 / 194 against 203, 30 steps 107 against 93 / 192 against 140; L = 48, one
+// step 116 against 133 / 217 against 334.
+static bool by_digits(int L, double flops) { return L >= 40 || flops >= 3e7; }
 
-emu_status emu_var_recursion(emu_ctx *ctx, const double *dXi, int n, int T, long ldxi, const double *dPhi, int P,
-                             double *dF, long ldf) {
-  if (!ctx || !dXi || !dF || n < 1 || T < 1 || ldxi < n || ldf < n || P < 0 || P > kMaxP || (P > 0 && !dPhi))
-    return EMU_EINVAL;
-  EMU_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
-  EMU_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, ST_WORDS * sizeof(int), ctx->stream));
-  k_var<<<(n + 127) / 128, 128, 0, ctx->stream>>>(dXi, ldxi, n, T, dPhi, P, dF, ldf, ctx->d_status);
-  EMU_LAUNCHED(ctx);
-  EMU_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
-  return EMU_OK;
-}
-
-emu_status emu_isht(emu_ctx *ctx, const double *dF, int L, int T, long ldf, int ntheta, int nphi, double *dZ,
-                    long ldz) {
-  if (!ctx || !dF || !dZ || L < 1 || L > 2048 || T < 1 || ldf < (long)L * L || ntheta < 2 || nphi < 1 ||
-      ldz < (long)ntheta * nphi)
-    return EMU_EINVAL;
-  EMU_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
+// The transforms' sums on the FP64 pipe: small transforms, operands with an
+// infinity or a NaN, and sizes whose digits do not fit the device.
+static emu_status isht_direct(emu_ctx *ctx, const double *dF, int L, int T, long ldf, int ntheta, int nphi, double *dZ,
+                              long ldz) {
   cudaStream_t s = ctx->stream;
-  EMU_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, ST_WORDS * sizeof(int), s));
   const size_t nlam = (size_t)ntheta * ((size_t)L * (L + 1) / 2);
   const long ldab = 2L * L * ntheta;
   double *lam = nullptr, *ab = nullptr, *cs = nullptr;
@@ -390,14 +382,9 @@ emu_status emu_isht(emu_ctx *ctx, const double *dF, int L, int T, long ldf, int 
 }
 
 
-emu_status emu_sht(emu_ctx *ctx, const double *dZ, int ntheta, int nphi, int T, long ldz, int L, double *dF,
-                   long ldf) {
-  if (!ctx || !dZ || !dF || L < 1 || L > 1024 || T < 1 || ntheta < 2 || nphi < 1 || ldz < (long)ntheta * nphi ||
-      ldf < (long)L * L)
-    return EMU_EINVAL;
-  EMU_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
+static emu_status sht_direct(emu_ctx *ctx, const double *dZ, int ntheta, int nphi, int T, long ldz, int L, double *dF,
+                             long ldf) {
   cudaStream_t s = ctx->stream;
-  EMU_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, ST_WORDS * sizeof(int), s));
   const int Q = 2 * L - 1, M = 2 * ntheta - 2;
   const size_t npair = (size_t)L * (L + 1) / 2;
   const long ldcs = 2L * L * ntheta;
@@ -408,9 +395,6 @@ emu_status emu_sht(emu_ctx *ctx, const double *dZ, int ntheta, int nphi, int T, 
   if (e == cudaSuccess) e = cudaMallocAsync(&sq, npair * 2 * Q * sizeof(double), s);
   if (e == cudaSuccess) e = cudaMallocAsync(&cs, (size_t)ldcs * T * sizeof(double), s);
   const size_t sm_S = (2 * (size_t)Q + ntheta) * sizeof(double), sm_K = (4 * (size_t)Q + ntheta) * sizeof(double);
-  if (e == cudaSuccess && (sm_S > 48 * 1024 || sm_K > 48 * 1024 || nphi * sizeof(double) > 48 * 1024)) {
-    e = cudaErrorInvalidValue;
-  }
   if (e == cudaSuccess) {
     ProfScope ps(ctx, PROF_SOLVE, 2.0 * (double)L * ntheta * nphi * T + 8.0 * (double)L * Q * M * T, 0.0);
     k_legendre<<<dim3((ntheta + 127) / 128, L), 128, 0, s>>>(L, ntheta, lam);
@@ -431,6 +415,55 @@ emu_status emu_sht(emu_ctx *ctx, const double *dZ, int ntheta, int nphi, int T, 
   return EMU_OK;
 }
 
+
+extern "C" {
+
+emu_status emu_var_recursion(emu_ctx *ctx, const double *dXi, int n, int T, long ldxi, const double *dPhi, int P,
+                             double *dF, long ldf) {
+  if (!ctx || !dXi || !dF || n < 1 || T < 1 || ldxi < n || ldf < n || P < 0 || P > kMaxP || (P > 0 && !dPhi))
+    return EMU_EINVAL;
+  EMU_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
+  EMU_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, ST_WORDS * sizeof(int), ctx->stream));
+  k_var<<<(n + 127) / 128, 128, 0, ctx->stream>>>(dXi, ldxi, n, T, dPhi, P, dF, ldf, ctx->d_status);
+  EMU_LAUNCHED(ctx);
+  EMU_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
+  return EMU_OK;
+}
+
+emu_status emu_isht(emu_ctx *ctx, const double *dF, int L, int T, long ldf, int ntheta, int nphi, double *dZ,
+                    long ldz) {
+  if (!ctx || !dF || !dZ || L < 1 || L > 2048 || T < 1 || ldf < (long)L * L || ntheta < 2 || nphi < 1 ||
+      ldz < (long)ntheta * nphi)
+    return EMU_EINVAL;
+  EMU_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
+  EMU_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, ST_WORDS * sizeof(int), ctx->stream));
+  const double flops = 2.0 * (double)L * L * ntheta * T + 4.0 * (double)L * ntheta * nphi * T;
+  if (by_digits(L, flops) && nphi <= 65535) {
+    ProfScope ps(ctx, PROF_SOLVE, flops, 0.0);
+    const emu_status s = isht_digits(ctx, dF, L, T, ldf, ntheta, nphi, dZ, ldz);
+    if (s != EMU_ENOMEM && s != EMU_ESTATE) return s;
+  }
+  return isht_direct(ctx, dF, L, T, ldf, ntheta, nphi, dZ, ldz);
+}
+
+emu_status emu_sht(emu_ctx *ctx, const double *dZ, int ntheta, int nphi, int T, long ldz, int L, double *dF,
+                   long ldf) {
+  if (!ctx || !dZ || !dF || L < 1 || L > 1024 || T < 1 || ntheta < 2 || nphi < 1 || ldz < (long)ntheta * nphi ||
+      ldf < (long)L * L)
+    return EMU_EINVAL;
+  // the shared memory of the direct sums bounds the sizes that are taken
+  const size_t Q = 2 * (size_t)L - 1;
+  if ((4 * Q + ntheta) * sizeof(double) > 48 * 1024 || nphi * sizeof(double) > 48 * 1024) return EMU_EINVAL;
+  EMU_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
+  EMU_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, ST_WORDS * sizeof(int), ctx->stream));
+  const double flops = 4.0 * (double)L * ntheta * nphi * T + 4.0 * (double)L * Q * ntheta * T;
+  if (by_digits(L, flops)) {
+    ProfScope ps(ctx, PROF_SOLVE, flops, 0.0);
+    const emu_status s = sht_digits(ctx, dZ, ntheta, nphi, T, ldz, L, dF, ldf);
+    if (s != EMU_ENOMEM && s != EMU_ESTATE) return s;
+  }
+  return sht_direct(ctx, dZ, ntheta, nphi, T, ldz, L, dF, ldf);
+}
 
 emu_status emu_emulate_grid(emu_ctx *ctx, const double *dZs, long G, int T, long ldz, const emu_trend *m,
                             const double *dsigma, const double *dv, uint64_t seed, uint32_t stream_id, double *dY,

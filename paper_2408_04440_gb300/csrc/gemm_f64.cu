@@ -28,6 +28,7 @@
 
 #include <algorithm>
 
+#include "digits.cuh"
 #include "gemm_f64.h"
 #include "gemm_tc.h"
 #include "tc.cuh"
@@ -135,7 +136,6 @@ __device__ inline void raise_timeout(Shared *sh, int *status) {
 // ------------------------------------------------------------- digits
 // 2^e for integer e in the normal range (exact).
 __device__ inline double exp2i(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
-__device__ inline int exp_of(const int *exps, long i) { return max(exps[i] - kExpBias, kExpMin); }
 // fixed_scaled for any s: near the ends of the FP64 range, and NaN where s
 // carries the poison of a row with an infinity or a NaN.
 __device__ __noinline__ double fixed_scaled_any(long long hi, unsigned lo, int s) {
@@ -143,70 +143,6 @@ __device__ __noinline__ double fixed_scaled_any(long long hi, unsigned lo, int s
   const double x = fma((double)hi, 0x1p-31, (double)lo * 0x1p-63);
   const int s1 = max(-1000, min(1000, s));
   return x * exp2i(s1) * exp2i(max(-1000, min(1000, s - s1)));
-}
-// Magnitude bits of x: ordered like |x|, infinities and then NaNs on top, so
-// that row maxima are taken in integers.
-__device__ inline unsigned long long mag_bits(double x) {
-  return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
-}
-// Biased exponent of a row whose largest magnitude bits are m > 0: every
-// |x| < 2^(result - kExpBias).  (The sign is masked again: the compiler takes
-// the mask above for an FP64 absolute value, which may keep a NaN's sign.)
-__device__ inline int biased_exp(unsigned long long m) {
-  const int ex = (int)(m >> 52) & 0x7ff;
-  if (ex == 0x7ff) return kExpPoison;
-  return (ex > 0 ? ex - 1022 : (64 - __clzll((long long)m)) - 1074) + kExpBias;
-}
-// x 2^(56 - e) rounded to the nearest integer (ties to even), for |x| < 2^e:
-// below 2^56 in magnitude.  In integer arithmetic on the significand: the FP64
-// pipe issues about one warp instruction per 19 cycles and SM, and a multiply
-// and a conversion per entry there took longer than the entry's memory traffic.
-// 0 where e is a poisoned row's.
-__device__ inline long long to_fixed(double x, int e) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  int ex = (int)(b >> 52) & 0x7ff;
-  unsigned long long m = b & 0xfffffffffffffull;
-  if (ex > 0) m |= 1ull << 52;
-  else ex = 1;
-  const int sh = ex - 1019 - e;  // x 2^(56 - e) = m 2^sh, sh <= 3
-  unsigned long long X;
-  if (sh >= 0) {
-    X = m << sh;
-  } else {
-    const int r = -sh < 54 ? -sh : 54;  // m < 2^53: 2^-54 m rounds to 0
-    X = (m + ((1ull << (r - 1)) - 1) + ((m >> r) & 1ull)) >> r;
-  }
-  return (long long)b < 0 ? -(long long)X : (long long)X;
-}
-
-// The NS digits of X (|X| <= 2^56, the unit of the last digit is 2^-56): peeled
-// off from the top, each rounded to nearest, so |digit 0| <= 128 and
-// |digit p| <= 64 for p >= 1 and sum_p digit_p 2^(7 (NS - 1 - p)) = X exactly.
-// As BF16 bits: a digit is at most eight bits wide, so the upper half of its
-// FP32 pattern (formed by an add of 1.5 2^23, no conversion) is exact.
-__device__ inline void digit_bits(long long X, uint32_t (&d)[NS]) {
-#pragma unroll
-  for (int p = 0; p < NS; p++) {
-    const int sh = SLICE_BITS * (NS - 1 - p);
-    const long long dg = (sh > 0) ? ((X + (1LL << (sh > 0 ? sh - 1 : 0))) >> sh) : X;
-    X -= dg << sh;
-    d[p] = __float_as_uint(__int_as_float(0x4B400000 + (int)dg) - 12582912.0f) >> 16;
-  }
-}
-// Digits of v with row exponent e written d[0], d[plane], ...
-__device__ inline void write_digits(double v, int e, uint16_t *d, size_t plane) {
-  uint32_t g[NS];
-  digit_bits(to_fixed(v, e), g);
-#pragma unroll
-  for (int p = 0; p < NS; p++) d[p * plane] = (uint16_t)g[p];
-}
-// The same for two neighbouring columns (d 4-byte aligned).
-__device__ inline void write_digits2(double v0, double v1, int e, uint16_t *d, size_t plane) {
-  uint32_t g0[NS], g1[NS];
-  digit_bits(to_fixed(v0, e), g0);
-  digit_bits(to_fixed(v1, e), g1);
-#pragma unroll
-  for (int p = 0; p < NS; p++) *reinterpret_cast<uint32_t *>(d + p * plane) = g0[p] | (g1[p] << 16);
 }
 // A 32 x 32 block (256 threads) in shared memory, row rr with exponent
 // exp(rr), to its digit planes at d + rr * ld: a half warp per row, two
@@ -532,9 +468,11 @@ __global__ void __launch_bounds__(256)
 constexpr int RG_W = 8;
 struct Work {
   long out_off;
+  int x;  // K offset in both arenas
   int a_sc, b_sc, rows_valid, cols_valid;
   int a_row, b_row;
   int total;  // K stages (0: nothing to do)
+  int m, row0, col0;  // batched and dense sources
 };
 // First row block of column group g.
 template <int SRC>
@@ -558,8 +496,60 @@ __host__ __device__ inline int region_items(const Region &rg) {
 struct Cursor {  // the group of the last item found; items come in ascending order
   int g = 0, base = 0;
 };
+// Items of the batched and dense sources.
+template <int SRC>
+__host__ __device__ inline int batch_items(const Region &rg) {
+  const int rb = ((SRC == SRC_DENSE ? rg.rows_valid : 2 * rg.T) + BM - 1) / BM;
+  if (SRC == SRC_DENSE) return rb * ((rg.cols_valid + BN - 1) / BN);
+  return rg.L * rb * (((SRC == SRC_SYN ? rg.ntheta : rg.L) + BN - 1) / BN);
+}
+template <int SRC>
+__device__ inline Work batch_work(const Region &rg, int it) {
+  const int rb = ((SRC == SRC_DENSE ? rg.rows_valid : 2 * rg.T) + BM - 1) / BM;
+  const int cb = ((SRC == SRC_DENSE ? rg.cols_valid : SRC == SRC_SYN ? rg.ntheta : rg.L) + BN - 1) / BN;
+  const int C = it % cb, R = it / cb % rb, m = it / cb / rb;
+  Work w;
+  w.out_off = 0;
+  w.x = 0;
+  w.a_row = w.a_sc = R * BM;
+  w.b_row = w.b_sc = C * BN;
+  w.m = m;
+  w.row0 = R * BM;
+  w.col0 = C * BN;
+  if (SRC == SRC_DENSE) {
+    w.total = rg.nk / BK;
+    w.rows_valid = rg.rows_valid - R * BM;
+    w.cols_valid = rg.cols_valid - C * BN;
+  } else if (SRC == SRC_SYN) {
+    w.total = order_k(rg.L, m) / BK;
+    w.x = order_koff(rg.L, m);
+    w.a_sc += m * rg.rpad;
+    w.b_sc += m * rg.cpad;
+    w.rows_valid = 2 * rg.T - R * BM;
+    w.cols_valid = rg.ntheta - C * BN;
+  } else {
+    w.total = rg.nk / BK;
+    w.a_row = w.a_sc = m * rg.rpad + R * BM;
+    w.b_row = w.b_sc = order_pos(rg.L, m) + C * BN;
+    w.rows_valid = 2 * rg.T - R * BM;
+    w.cols_valid = rg.L - m - C * BN;
+    if (w.cols_valid <= 0) w.total = 0;
+  }
+  return w;
+}
+// Output offset of row `row` of an item's block, and of column cx.
+template <int SRC>
+__device__ inline long batch_row(const Region &rg, const Work &w, int row, long ldo) {
+  const int r = w.row0 + row;
+  if (SRC == SRC_DENSE) return (long)(r / rg.div) * rg.ld2 + r % rg.div + (long)w.col0 * ldo;
+  const int s = r / rg.T, t = r - s * rg.T;
+  if (SRC == SRC_SYN) return t + (long)rg.T * (w.col0 + (long)rg.ntheta * (2 * w.m + s));
+  return t * ldo;
+}
+
 template <int SRC>
 __device__ inline Work region_work(const Region &rg, Cursor &cur, int it, long ldo) {
+  if constexpr (SRC >= SRC_DENSE) return batch_work<SRC>(rg, it);
   int cnt;
   while (it >= cur.base + (cnt = group_items<SRC>(rg, cur.g))) {
     cur.base += cnt;
@@ -572,6 +562,7 @@ __device__ inline Work region_work(const Region &rg, Cursor &cur, int it, long l
   w.rows_valid = BM;
   w.cols_valid = BN;
   w.total = nb / BK;
+  w.x = 0;
   if (SRC == SRC_SYRK) {
     if (row + BM - 1 < col) w.total = 0;  // above the diagonal
     w.out_off = tile_index(row / nb, col / nb, rg.NT) * (long)nb * nb + row % nb + (long)(col % nb) * nb;
@@ -653,7 +644,7 @@ __global__ void __maxnreg__(96)
           kst = wk.total;
           sd.a_row = wk.a_row;
           sd.b_row = wk.b_row;
-          sd.a_x = sd.b_x = 0;
+          sd.a_x = sd.b_x = wk.x;
         }
         for (int sg = sg0; sg < sg1 && ok; sg++) {
           if constexpr (SRC == SRC_LIST) sd = segs[sg];
@@ -776,7 +767,11 @@ __global__ void __maxnreg__(96)
       const int total = item.total;
       const int nchunks = (total + CHUNK_STAGES - 1) / CHUNK_STAGES;
       constexpr bool kWhole = MODE == TC64_SUB;  // every row and column exists
-      double *o = out + item.out_off + row;
+      double *o = out + item.out_off;
+      if constexpr (SRC >= SRC_DENSE)
+        o += batch_row<SRC>(rg, item, row, ldo);
+      else
+        o += row;
       if constexpr (kWhole) {
         // the warp's 32 rows x EC columns (two 128-byte lines per column) on
         // their way to L2 while the MMAs run
@@ -832,8 +827,16 @@ __global__ void __maxnreg__(96)
             double v = fixed_scaled(hi[x0 + x], lo[x0 + x], ea + exp_of(b_exp, (long)item.b_sc + cx));
             if (MODE == TC64_SUB)
               __stcg(o + (long)cx * ldo, cv[x] - v);
-            else if (kWhole || cx < item.cols_valid)
-              __stcg(o + (long)cx * ldo, MODE == TC64_SET ? v : cv[x] + v);
+            else if (kWhole || cx < item.cols_valid) {
+              if constexpr (SRC == SRC_ANA) {
+                // order +-m, degree l = m + column; the sine sums of order 0 have no coefficient
+                const long l = item.m + item.col0 + cx;
+                const bool neg = item.row0 + row >= rg.T;
+                if (!neg || item.m > 0) __stcg(o + l * l + l + (neg ? -item.m : item.m), v);
+              } else {
+                __stcg(o + (long)cx * ldo, MODE == TC64_SET ? v : cv[x] + v);
+              }
+            }
           }
         }
       }
@@ -957,15 +960,22 @@ emu_status launch(emu_ctx *ctx, const CUtensorMap &a, const CUtensorMap &b, cons
 emu_status launch_region(emu_ctx *ctx, int src, const CUtensorMap &a, const CUtensorMap &b, const Region &rg,
                          int a_plane, int b_plane, const int *a_exp, const int *b_exp, double *out, long ldo,
                          int max_ctas) {
-  if (rg.nb % BM != 0) return EMU_EINVAL;
-  const int n = src == SRC_SYRK ? region_items<SRC_SYRK>(rg) : region_items<SRC_TRMM>(rg);
+  if (src < SRC_DENSE && rg.nb % BM != 0) return EMU_EINVAL;
+  const int n = src == SRC_SYRK    ? region_items<SRC_SYRK>(rg)
+                : src == SRC_DENSE ? batch_items<SRC_DENSE>(rg)
+                : src == SRC_SYN   ? batch_items<SRC_SYN>(rg)
+                : src == SRC_ANA   ? batch_items<SRC_ANA>(rg)
+                                   : region_items<SRC_TRMM>(rg);
   if (n <= 0) return EMU_OK;
   const int grid = std::max(1, std::min(n, max_ctas));
 #define EMU_REGION(M, S) \
   launch_kernel<M, S>(ctx, grid, a, b, nullptr, n, nullptr, rg.nb, a_plane, b_plane, a_exp, b_exp, out, ldo, rg)
   if (src == SRC_SYRK) return EMU_REGION(TC64_SUB, SRC_SYRK);
   if (src == SRC_TRSM) return EMU_REGION(TC64_SUB, SRC_TRSM);
-  return EMU_REGION(TC64_SET, SRC_TRMM);
+  if (src == SRC_TRMM) return EMU_REGION(TC64_SET, SRC_TRMM);
+  if (src == SRC_DENSE) return EMU_REGION(TC64_SET, SRC_DENSE);
+  if (src == SRC_SYN) return EMU_REGION(TC64_SET, SRC_SYN);
+  return EMU_REGION(TC64_SET, SRC_ANA);
 #undef EMU_REGION
 }
 

@@ -122,15 +122,47 @@ struct Region {
   const int *tiles = nullptr;  // TRSM: tile indices; tile z has slot slot0 + z
   int slot0 = 0;
   int a_row0 = 0;            // TRMM: matrix row held by arena row 0 of A
-  int rows_valid = 0, cols_valid = 0;  // TRMM: rows / columns of the output that exist
+  int rows_valid = 0, cols_valid = 0;  // TRMM, DENSE: rows / columns of the output that exist
+  int nk = 0;                // DENSE, ANA: K (a multiple of BK)
+  int div = 0;               // DENSE
+  long ld2 = 0;              // DENSE
+  int L = 0, T = 0, ntheta = 0;  // SYN, ANA
+  int rpad = 0, cpad = 0;    // SYN, ANA: rows of A per order (SYN: exponents only), SYN: rows of B
 };
+// SYN operands: the orders run in blocks of 32 from m0; order m's K holds the
+// degrees m0 .. L-1 (zero below m), order_k(L, m) of them (a multiple of 32),
+// from K offset order_koff(L, m).
+__host__ __device__ inline int order_k(int L, int m) { return (L + 31) / 32 * 32 - m / 32 * 32; }
+__host__ __device__ inline int order_koff(int L, int m) {
+  const int Lp = (L + 31) / 32 * 32, b = m / 32;
+  return 32 * (b * Lp - 16 * b * (b - 1)) + (m % 32) * (Lp - 32 * b);
+}
+// ANA operands: the (m, l) pairs of even orders, then from order_odd0(L) on
+// those of odd orders (the two parities are formed by different products, in
+// blocks of BM rows); order m's pairs start at order_pos(L, m), l = m first.
+__host__ __device__ inline int order_odd0(int L) {
+  const int a = (L + 1) / 2;
+  return (a * L - a * (a - 1) + 127) / 128 * 128;
+}
+__host__ __device__ inline int order_pos(int L, int m) {
+  const int a = m / 2;
+  return m % 2 == 0 ? a * L - a * (a - 1) : order_odd0(L) + a * L - a * a;
+}
 // SYRK: out = t64: tiles (r, c) -= A_r B_c^T for the blocks of the region on
 //   or below the diagonal; A and B rows are matrix rows of a panel's digits.
 // TRSM: out = t64: column block c of the listed tiles -= X_J L_cJ^T; X digits
 //   per slot (launch_trsm_block), L_kk digits of block J (launch_lkk_digits).
 // TRMM: out(row, col) = A_row B_col^T over K = the row's tiles 0 .. row / nb,
 //   out column-major; A rows start at matrix row a_row0.
-enum { SRC_LIST = 0, SRC_SYRK = 1, SRC_TRSM = 2, SRC_TRMM = 3 };
+// DENSE: rows r < rows_valid (K-major digits), columns c < cols_valid, K = nk:
+//   out[(r / div) * ld2 + r % div + c * ldo].
+// SYN, per order m < L (of a spherical-harmonic transform): rows (s, t) = s T + t
+//   (s = 0: order m, 1: order -m), columns i < ntheta, K the degrees of m's
+//   block of 32 orders (order_k); out[t + T (i + ntheta (2 m + s)).
+// ANA, per order m < L: rows (s, t), columns l - m for l = m .. L-1, K = nk
+//   grid rings; A rows m rpad + (s, t), B rows order_pos(m) + l - m;
+//   out[t ldo + l^2 + l +- m].
+enum { SRC_LIST = 0, SRC_SYRK = 1, SRC_TRSM = 2, SRC_TRMM = 3, SRC_DENSE = 4, SRC_SYN = 5, SRC_ANA = 6 };
 emu_status launch_region(emu_ctx *ctx, int src, const CUtensorMap &a, const CUtensorMap &b, const Region &rg,
                          int a_plane, int b_plane, const int *a_exp, const int *b_exp, double *out, long ldo,
                          int max_ctas);
