@@ -394,12 +394,15 @@ __global__ void __launch_bounds__(256) k_sigma_apply(int L, int n, int nb, const
 
 // Gaussian probes G (n_pad x p, zero beyond n) from the library's normals.
 __global__ void k_probes(uint64_t seed, int n, long npad, int p, double *__restrict__ G, long ldg) {
+  __shared__ NormalTables T;
+  T.load();
+  __syncthreads();
   const long npairs = (npad + 1) / 2;
   for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < npairs * p; q += (long)gridDim.x * blockDim.x) {
     const long pr = q % npairs;
     const int col = (int)(q / npairs);
-    double z[2] = {0.0, 0.0};
-    normal_pair(seed, 7u, pr, col, (int)npad, z);
+    const double2 v = normal_pair(seed, 7u, pr, col, T);
+    const double z[2] = {v.x, v.y};
     for (int u = 0; u < 2; u++) {
       const long r = 2 * pr + u;
       if (r < npad) G[r + (size_t)col * ldg] = r < n ? z[u] : 0.0;

@@ -279,33 +279,43 @@ __global__ void k_sht_contract(int L, int T, int ntheta, const double *__restric
 // years before the trajectory at x[0]: D_1 = x[0], D_(y+1) = (1 - rho) x_y + rho D_y.
 // One thread per grid-point pair (the two rows of one Box-Muller pair) and
 // chunk of kEmTC time steps (blockIdx.y); the harmonic values of the chunk
-// are shared by the block.  HBM-bound: 16 bytes in, 8 out per entry.
+// are shared by the block.  Bound by FP64 issue: 32 instructions of a normal
+// pair and 2 K + 2 per entry.
 constexpr int kMaxK = 8, kEmTC = 32;
 struct TrendDev {
   int K, nyears;
   double tau;
   const double *b0, *b1, *b2, *rho, *a, *b, *x;
 };
-__global__ void __launch_bounds__(128) k_emulate_grid(const double *__restrict__ Zs, long G, int T, long ldz,
-                                                      TrendDev m, const double *__restrict__ sigma,
+// KM: harmonic pairs held in registers (0, 4 or 8; those from K on are zeros).
+// vec: 16-byte aligned columns.
+template <int KM>
+__global__ void __launch_bounds__(128) k_emulate_grid(const double *Zs, long G, int T, long ldz, TrendDev m,
+                                                      const double *__restrict__ sigma,
                                                       const double *__restrict__ v, uint64_t seed, uint32_t sid,
-                                                      double *Y, long ldy) {
-  __shared__ double cs[kMaxK][kEmTC], sn[kMaxK][kEmTC];
+                                                      double *Y, long ldy, bool vec) {
+  __shared__ double cs[KM + 1][kEmTC], sn[KM + 1][kEmTC];
+  __shared__ int yr[kEmTC];  // forcing years of the chunk's steps
+  __shared__ NormalTables tab;
+  tab.load();
   const int t0 = blockIdx.y * kEmTC + 1;
   const int nt = min(kEmTC, T - t0 + 1);
   const double two_pi = 6.283185307179586476925286766559;
-  for (int q = threadIdx.x; q < m.K * kEmTC; q += blockDim.x) {
+  for (int q = threadIdx.x; q < KM * kEmTC; q += blockDim.x) {
     int k = q / kEmTC + 1, tt = q % kEmTC;
     sincos(two_pi * (double)(t0 + tt) * (double)k / m.tau, &sn[k - 1][tt], &cs[k - 1][tt]);
   }
+  if (threadIdx.x < kEmTC) yr[threadIdx.x] = (int)ceil((double)(t0 + threadIdx.x) / m.tau);
   __syncthreads();
   const long p = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (2 * p >= G) return;
-  const int npt = (2 * p + 1 < G) ? 2 : 1;
-  double b0[2], b1[2], b2[2], rho[2], sg[2], vv[2], D[2], a[2][kMaxK], b[2][kMaxK];
-  long yc = (long)ceil((double)t0 / m.tau);  // forcing year of the chunk's first step
+  const bool two = 2 * p + 1 < G;
+  // trend without its harmonics, renewed when the forcing year changes
+  double b0[2], b1[2], b2[2], rho[2], sg[2], vv[2], D[2], base[2], a[2][KM + 1], b[2][KM + 1];
+  long yc = 0;
+#pragma unroll
   for (int u = 0; u < 2; u++) {
-    long g = 2 * p + (u < npt ? u : 0);
+    const long g = 2 * p + (two ? u : 0);
     b0[u] = m.b0[g];
     b1[u] = m.b1[g];
     b2[u] = m.b2[g];
@@ -313,29 +323,51 @@ __global__ void __launch_bounds__(128) k_emulate_grid(const double *__restrict__
     sg[u] = sigma[g];
     vv[u] = v[g];
 #pragma unroll
-    for (int k = 0; k < kMaxK; k++) {
+    for (int k = 0; k < KM; k++) {
       a[u][k] = k < m.K ? m.a[k + g * m.K] : 0.0;
       b[u][k] = k < m.K ? m.b[k + g * m.K] : 0.0;
     }
     D[u] = m.x[0];
-    for (long yy = 1; yy < yc; yy++) D[u] = (1.0 - rho[u]) * m.x[yy] + rho[u] * D[u];
+    base[u] = 0.0;
   }
   for (int tt = 0; tt < nt; tt++) {
     const int t = t0 + tt;
-    const long y = (long)ceil((double)t / m.tau);
-    while (yc < y) {
-      for (int u = 0; u < 2; u++) D[u] = (1.0 - rho[u]) * m.x[yc] + rho[u] * D[u];
-      yc++;
+    const long y = yr[tt];
+    if (yc < y) {
+      // D of year y from D of year max(yc, 1)
+      for (yc = yc > 0 ? yc : 1; yc < y; yc++)
+#pragma unroll
+        for (int u = 0; u < 2; u++) D[u] = (1.0 - rho[u]) * m.x[yc] + rho[u] * D[u];
+      const double xy = m.x[y];
+#pragma unroll
+      for (int u = 0; u < 2; u++) base[u] = b0[u] + b1[u] * xy + b2[u] * D[u];
     }
-    double e[2] = {0.0, 0.0};
-    normal_pair(seed, sid, p, t - 1, (int)(G < 0x7fffffff ? G : 0x7fffffff), e);
-    const double xy = m.x[y];
-    for (int u = 0; u < npt; u++) {
-      double mt = b0[u] + b1[u] * xy + b2[u] * D[u];
-      for (int k = 0; k < m.K; k++) mt += a[u][k] * cs[k][tt] + b[u][k] * sn[k][tt];
-      const long g = 2 * p + u;
-      const double z = Zs[g + (long)(t - 1) * ldz] + vv[u] * e[u];
-      Y[g + (long)(t - 1) * ldy] = mt + sg[u] * z;
+    const double2 ep = normal_pair(seed, sid, p, t - 1, tab);
+    const double e[2] = {ep.x, ep.y};
+    const double *zp = Zs + 2 * p + (long)(t - 1) * ldz;
+    double *yp = Y + 2 * p + (long)(t - 1) * ldy;
+    double z[2], o[2];
+    if (vec && two) {
+      const double2 zz = *reinterpret_cast<const double2 *>(zp);
+      z[0] = zz.x;
+      z[1] = zz.y;
+    } else {
+      z[0] = zp[0];
+      z[1] = two ? zp[1] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      double mt = base[u];
+#pragma unroll
+      for (int k = 0; k < KM; k++)
+        if (KM <= 4 || k < m.K) mt = fma(a[u][k], cs[k][tt], fma(b[u][k], sn[k][tt], mt));
+      o[u] = fma(sg[u], fma(vv[u], e[u], z[u]), mt);
+    }
+    if (vec && two) {
+      *reinterpret_cast<double2 *>(yp) = make_double2(o[0], o[1]);
+    } else {
+      yp[0] = o[0];
+      if (two) yp[1] = o[1];
     }
   }
 }
@@ -482,7 +514,10 @@ emu_status emu_emulate_grid(emu_ctx *ctx, const double *dZs, long G, int T, long
   dim3 grid((unsigned)((pairs + 127) / 128), (unsigned)((T + kEmTC - 1) / kEmTC));
   {
     ProfScope ps(ctx, PROF_RNG, 0.0, 24.0 * (double)G * T);
-    k_emulate_grid<<<grid, 128, 0, ctx->stream>>>(dZs, G, T, ldz, td, dsigma, dv, seed, stream_id, dY, ldy);
+    const bool vec = ldz % 2 == 0 && ldy % 2 == 0 &&
+                     ((reinterpret_cast<uintptr_t>(dZs) | reinterpret_cast<uintptr_t>(dY)) & 15) == 0;
+    auto kern = m->K == 0 ? k_emulate_grid<0> : m->K <= 4 ? k_emulate_grid<4> : k_emulate_grid<kMaxK>;
+    kern<<<grid, 128, 0, ctx->stream>>>(dZs, G, T, ldz, td, dsigma, dv, seed, stream_id, dY, ldy, vec);
     EMU_LAUNCHED(ctx);
   }
   EMU_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));

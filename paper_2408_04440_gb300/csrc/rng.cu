@@ -12,55 +12,65 @@
 
 namespace {
 
-__global__ void k_normals(uint64_t seed, uint32_t stream_id, int nrows, int s,
-                          double *__restrict__ Z, long ldz) {
-  long npairs = (nrows + 1) / 2;
-  long total = npairs * s;
-  for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < total;
-       q += (long)gridDim.x * blockDim.x) {
-    long p = q % npairs;
-    int col = (int)(q / npairs);
-    normal_pair(seed, stream_id, p, col, nrows, Z + (size_t)col * ldz + 2 * p);
-  }
+// Pairs on x, columns on y; nrows is even when `vec` (16-byte stores).
+__global__ void __launch_bounds__(256)
+    k_normals(uint64_t seed, uint32_t stream_id, int nrows, int s, double *__restrict__ Z, long ldz, bool vec) {
+  __shared__ NormalTables T;
+  T.load();
+  __syncthreads();
+  const int npairs = (nrows + 1) / 2;
+  for (int col = blockIdx.y; col < s; col += gridDim.y)
+    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < npairs; p += gridDim.x * blockDim.x) {
+      const double2 v = normal_pair(seed, stream_id, p, col, T);
+      double *z = Z + (size_t)col * ldz + 2L * p;
+      if (vec) {
+        *reinterpret_cast<double2 *>(z) = v;
+      } else {
+        z[0] = v.x;
+        if (2L * p + 1 < nrows) z[1] = v.y;
+      }
+    }
 }
 
 // Batch: blockIdx.y = matrix b, all NT_b * nb padded rows of its block of the
 // stacked Z (rows row_base ..), with its own stream id.
 // The seed is read from device memory so that a captured graph can be
 // replayed with another seed.
-__global__ void k_normals_batch(const uint64_t *__restrict__ seed_p, const BatchInst *__restrict__ inst, int nb,
+__global__ void __launch_bounds__(256)
+    k_normals_batch(const uint64_t *__restrict__ seed_p, const BatchInst *__restrict__ inst, int nb,
                                 int s, double *__restrict__ Z, long ldz) {
+  __shared__ NormalTables T;
+  T.load();
+  __syncthreads();
   const uint64_t seed = *seed_p;
-  BatchInst I = inst[blockIdx.y];
-  int nrows = I.NT * nb;
-  long npairs = (nrows + 1) / 2;
-  long total = npairs * s;
+  const BatchInst I = inst[blockIdx.y];
+  const int npairs = I.NT * nb / 2;  // nb is even
   double *Zb = Z + I.row_base;
-  for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < total; q += (long)gridDim.x * blockDim.x) {
-    long p = q % npairs;
-    int col = (int)(q / npairs);
-    normal_pair(seed, (uint32_t)I.stream_id, p, col, nrows, Zb + (size_t)col * ldz + 2 * p);
-  }
+  for (int col = blockIdx.x; col < s; col += gridDim.x)
+    for (int p = threadIdx.x; p < npairs; p += blockDim.x)
+      *reinterpret_cast<double2 *>(Zb + (size_t)col * ldz + 2L * p) =
+          normal_pair(seed, (uint32_t)I.stream_id, p, col, T);
 }
 }  // namespace
 
 emu_status launch_normals(emu_ctx *ctx, uint64_t seed, uint32_t stream_id, int nrows,
                           int s, double *Z, long ldz) {
-  long total = (long)((nrows + 1) / 2) * s;
-  long blocks = (total + 255) / 256;
-  if (blocks > 8L * ctx->sm_count) blocks = 8L * ctx->sm_count;
-  if (blocks < 1) blocks = 1;
+  // about eight CTAs per SM, each with pairs enough to pay for its 11 KB of tables
+  const int most = std::max(1, ((nrows + 1) / 2 + 255) / 256);
+  const int gy = std::max(1, std::min(s, 8 * ctx->sm_count));
+  const int gx = std::max(1, std::min(most, 8 * ctx->sm_count / gy));
+  const bool vec = nrows % 2 == 0 && ldz % 2 == 0 && (reinterpret_cast<uintptr_t>(Z) & 15) == 0;
   ProfScope ps(ctx, PROF_RNG, 0.0, 8.0 * nrows * (double)s);
-  k_normals<<<(unsigned)blocks, 256, 0, ctx->stream>>>(seed, stream_id, nrows, s, Z, ldz);
+  k_normals<<<dim3(gx, gy), 256, 0, ctx->stream>>>(seed, stream_id, nrows, s, Z, ldz, vec);
   EMU_LAUNCHED(ctx);
   return EMU_OK;
 }
 
 emu_status launch_normals_batch(emu_ctx *ctx, const uint64_t *d_seed, const BatchInst *d_inst, int count,
                                 int maxNT, int nb, int s, double *Z, long ldz) {
-  long per = (long)((maxNT * nb + 1) / 2) * s;
-  int bx = (int)std::min<long>(std::max<long>((per + 255) / 256, 1), 64);
+  const int bx = std::max(1, std::min(s, 16));
   ProfScope ps(ctx, PROF_RNG, 0.0, 0.0);
+  if (ldz % 2 != 0) return EMU_EINVAL;
   k_normals_batch<<<dim3(bx, count), 256, 0, ctx->stream>>>(d_seed, d_inst, nb, s, Z, ldz);
   EMU_LAUNCHED(ctx);
   return EMU_OK;
