@@ -718,12 +718,6 @@ extern "C" emu_status emu_sample_host(emu_ctx *ctx, const emu_mat *L, int nsampl
 }
 
 // ------------------------------------------------------------------ solves
-// Copies B (n rows) into a zero-padded npad-row buffer, solves there.
-static emu_status potrs_padded(emu_ctx *ctx, const emu_mat *L, double *X, long ldx, int nrhs) {
-  if (L->state == MAT_FACTOR64) return launch_potrs64(ctx, L, X, ldx, nrhs);
-  return mixed_potrs(ctx, L, X, ldx, nrhs);
-}
-
 extern "C" emu_status emu_potrs(emu_ctx *ctx, const emu_mat *L, const double *dB, long ldb,
                                 double *dX, long ldx, int nrhs) {
   if (!ctx || !L || !dB || !dX || nrhs < 0 || ldb < L->n || ldx < L->n) return EMU_EINVAL;
@@ -739,7 +733,7 @@ extern "C" emu_status emu_potrs(emu_ctx *ctx, const emu_mat *L, const double *dB
   if (e == cudaSuccess)
     e = cudaMemcpy2DAsync(W, npad * sizeof(double), dB, ldb * sizeof(double),
                           (size_t)L->n * sizeof(double), nrhs, cudaMemcpyDeviceToDevice, ctx->stream);
-  emu_status s = (e == cudaSuccess) ? potrs_padded(ctx, L, W, npad, nrhs) : emu_cuda_fail(ctx, e, "potrs copy-in");
+  emu_status s = (e == cudaSuccess) ? factor_potrs(ctx, L, W, npad, nrhs) : emu_cuda_fail(ctx, e, "potrs copy-in");
   if (s == EMU_OK) {
     e = cudaMemcpy2DAsync(dX, ldx * sizeof(double), W, npad * sizeof(double),
                           (size_t)L->n * sizeof(double), nrhs, cudaMemcpyDeviceToDevice, ctx->stream);

@@ -248,8 +248,6 @@ emu_status launch_tril_diag(emu_ctx *ctx, emu_mat *A);
 emu_status launch_trmm64(emu_ctx *ctx, const emu_mat *L, const double *Z,
                          long ldz, int s, double *Y, long ldy,
                          const unsigned char *cls = nullptr);
-emu_status launch_potrs64(emu_ctx *ctx, const emu_mat *L, double *X, long ldx,
-                          int nrhs);
 // rng.cu
 emu_status launch_normals(emu_ctx *ctx, uint64_t seed, uint32_t stream_id,
                           int nrows, int s, double *Z, long ldz);

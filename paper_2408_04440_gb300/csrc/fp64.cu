@@ -1,7 +1,7 @@
 // fp64.cu -- FP64 kernels of the tile Cholesky ("Advancements in Dense Linear
 // Algebra": POTRF on the diagonal tile, TRSM on the panel, SYRK/GEMM on the
 // trailing tiles), the TRMM that draws emulations ("Generating Emulations",
-// xi = V z) and the tile-blocked triangular solves.
+// xi = V z).
 //
 // GB300 runs FP64 on the SIMT pipe at about 2 DFMA per clock per SM (the FP64
 // MMA path measured slower), so these kernels are FP64-issue bound: the
@@ -1656,72 +1656,6 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// -------------------------------------------------- triangular solves
-// Block-row update of the forward solve: X_k -= sum_{j<k} L_kj X_j, and of
-// the backward solve: X_k -= sum_{i>k} L_ik^T X_i.  One thread per (row,
-// rhs); the sums run over tiles in a fixed order.
-__global__ void k_solve_update(const double *__restrict__ t64, int nb, int NT, int k,
-                               int backward, double *__restrict__ X, long ldx, int nrhs) {
-  int r = blockIdx.x * blockDim.x + threadIdx.x;
-  int c = blockIdx.y;
-  if (r >= nb) return;
-  double acc = 0.0;
-  if (!backward) {
-    for (int j = 0; j < k; j++) {
-      const double *T = t64 + (size_t)tile_index(k, j, NT) * nb * nb;
-      const double *xj = X + (size_t)j * nb + (size_t)c * ldx;
-      for (int p = 0; p < nb; p++) acc += T[r + (size_t)p * nb] * xj[p];
-    }
-  } else {
-    for (int i = k + 1; i < NT; i++) {
-      const double *T = t64 + (size_t)tile_index(i, k, NT) * nb * nb;
-      const double *xi = X + (size_t)i * nb + (size_t)c * ldx;
-      for (int p = 0; p < nb; p++) acc += T[p + (size_t)r * nb] * xi[p];
-    }
-  }
-  X[(size_t)k * nb + r + (size_t)c * ldx] -= acc;
-}
-
-// Solve with the diagonal tile: one CTA per right-hand side, one thread per
-// row; column-oriented substitution (L x = b) or row-oriented (L^T x = b).
-__global__ void k_solve_diag(const double *__restrict__ t64, int nb, int NT, int k,
-                             int backward, double *__restrict__ X, long ldx) {
-  extern __shared__ double xs[];
-  int c = blockIdx.x;
-  const double *D = t64 + (size_t)tile_index(k, k, NT) * nb * nb;
-  double *x = X + (size_t)k * nb + (size_t)c * ldx;
-  for (int r = threadIdx.x; r < nb; r += blockDim.x) xs[r] = x[r];
-  __syncthreads();
-  if (!backward) {
-    for (int p = 0; p < nb; p++) {
-      double xp = xs[p] / D[p + (size_t)p * nb];
-      __syncthreads();
-      if (threadIdx.x == 0) xs[p] = xp;
-      for (int r = p + 1 + threadIdx.x; r < nb; r += blockDim.x)
-        xs[r] -= D[r + (size_t)p * nb] * xp;
-      __syncthreads();
-    }
-  } else {
-    for (int p = nb - 1; p >= 0; p--) {
-      // x_p = (y_p - sum_{r>p} L[r,p] x_r) / L[p,p]: reduce over r
-      double part = 0.0;
-      for (int r = p + 1 + threadIdx.x; r < nb; r += blockDim.x)
-        part += D[r + (size_t)p * nb] * xs[r];
-      __shared__ double red[32];
-      for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
-      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        double sum = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) sum += red[w];
-        xs[p] = (xs[p] - sum) / D[p + (size_t)p * nb];
-      }
-      __syncthreads();
-    }
-  }
-  for (int r = threadIdx.x; r < nb; r += blockDim.x) x[r] = xs[r];
-}
-
 }  // namespace
 
 extern "C" emu_status emu_potrf_task_list(int nb, int single_tile, int16_t *h_tasks, size_t max_tasks,
@@ -1956,31 +1890,5 @@ emu_status launch_trmm64(emu_ctx *ctx, const emu_mat *L, const double *Z, long l
   ProfScope ps(ctx, PROF_TRMM64, (double)L->n * L->n * s, 8.0 * tile_count(L->nt) * L->nb * L->nb);
   k_trmm64<<<grid, 256, 0, ctx->stream>>>(L->t64, L->n, L->nb, L->nt, Z, ldz, s, Y, ldy, cls);
   EMU_LAUNCHED(ctx);
-  return EMU_OK;
-}
-
-// X (npad x nrhs, ld ldx >= npad, padded rows zero) <- (L L^T)^{-1} X.
-emu_status launch_potrs64(emu_ctx *ctx, const emu_mat *L, double *X, long ldx, int nrhs) {
-  int nb = L->nb, NT = L->nt;
-  int thr = 256;
-  ProfScope ps(ctx, PROF_SOLVE, 2.0 * L->n * L->n * nrhs, 16.0 * tile_count(NT) * nb * nb);
-  for (int k = 0; k < NT; k++) {
-    if (k > 0) {
-      k_solve_update<<<dim3((nb + thr - 1) / thr, nrhs), thr, 0, ctx->stream>>>(
-          L->t64, nb, NT, k, 0, X, ldx, nrhs);
-      EMU_LAUNCHED(ctx);
-    }
-    k_solve_diag<<<nrhs, 512, nb * sizeof(double), ctx->stream>>>(L->t64, nb, NT, k, 0, X, ldx);
-    EMU_LAUNCHED(ctx);
-  }
-  for (int k = NT - 1; k >= 0; k--) {
-    if (k < NT - 1) {
-      k_solve_update<<<dim3((nb + thr - 1) / thr, nrhs), thr, 0, ctx->stream>>>(
-          L->t64, nb, NT, k, 1, X, ldx, nrhs);
-      EMU_LAUNCHED(ctx);
-    }
-    k_solve_diag<<<nrhs, 512, nb * sizeof(double), ctx->stream>>>(L->t64, nb, NT, k, 1, X, ldx);
-    EMU_LAUNCHED(ctx);
-  }
   return EMU_OK;
 }

@@ -371,73 +371,6 @@ __global__ void k_split_z(const double *__restrict__ Z, long ldz, long npad, int
   }
 }
 
-// ---------------------------------------------- FP32 triangular solves
-// Tile element (r, c) of a factor tile in FP32: diagonal and FP64-class tiles
-// from t64, others from the FP32 master.
-__device__ inline float ftile(const double *t64, const float *t32, const unsigned char *cls, long t, int nb,
-                              int r, int c, bool diag) {
-  size_t o = (size_t)t * nb * nb + r + (size_t)c * nb;
-  return (diag || cls[t] == EMU_CLASS_FP64) ? (float)t64[o] : t32[o];
-}
-
-__global__ void k_solve32_update(const double *__restrict__ t64, const float *__restrict__ t32,
-                                 const unsigned char *__restrict__ cls, int nb, int NT, int k, int backward,
-                                 double *__restrict__ X, long ldx) {
-  int r = blockIdx.x * blockDim.x + threadIdx.x;
-  int c = blockIdx.y;
-  if (r >= nb) return;
-  float acc = 0.f;
-  if (!backward) {
-    for (int j = 0; j < k; j++) {
-      long t = tile_index(k, j, NT);
-      const double *xj = X + (size_t)j * nb + (size_t)c * ldx;
-      for (int p = 0; p < nb; p++) acc += ftile(t64, t32, cls, t, nb, r, p, false) * (float)xj[p];
-    }
-  } else {
-    for (int i = k + 1; i < NT; i++) {
-      long t = tile_index(i, k, NT);
-      const double *xi = X + (size_t)i * nb + (size_t)c * ldx;
-      for (int p = 0; p < nb; p++) acc += ftile(t64, t32, cls, t, nb, p, r, false) * (float)xi[p];
-    }
-  }
-  X[(size_t)k * nb + r + (size_t)c * ldx] -= (double)acc;
-}
-
-__global__ void k_solve32_diag(const double *__restrict__ t64, int nb, int NT, int k, int backward,
-                               double *__restrict__ X, long ldx) {
-  extern __shared__ float xs[];
-  __shared__ float red[32];
-  int c = blockIdx.x;
-  const double *D = t64 + (size_t)tile_index(k, k, NT) * nb * nb;
-  double *x = X + (size_t)k * nb + (size_t)c * ldx;
-  for (int r = threadIdx.x; r < nb; r += blockDim.x) xs[r] = (float)x[r];
-  __syncthreads();
-  if (!backward) {
-    for (int p = 0; p < nb; p++) {
-      float xp = xs[p] / (float)D[p + (size_t)p * nb];
-      __syncthreads();
-      if (threadIdx.x == 0) xs[p] = xp;
-      for (int r = p + 1 + threadIdx.x; r < nb; r += blockDim.x) xs[r] -= (float)D[r + (size_t)p * nb] * xp;
-      __syncthreads();
-    }
-  } else {
-    for (int p = nb - 1; p >= 0; p--) {
-      float part = 0.f;
-      for (int r = p + 1 + threadIdx.x; r < nb; r += blockDim.x) part += (float)D[r + (size_t)p * nb] * xs[r];
-      for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
-      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        float sum = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) sum += red[w];
-        xs[p] = (xs[p] - sum) / (float)D[p + (size_t)p * nb];
-      }
-      __syncthreads();
-    }
-  }
-  for (int r = threadIdx.x; r < nb; r += blockDim.x) x[r] = (double)xs[r];
-}
-
 }  // namespace
 
 // ------------------------------------------------------------------ plan
@@ -1521,33 +1454,6 @@ emu_status mixed_sample(emu_ctx *ctx, const emu_mat *L, const double *Z, long ld
   // the host vectors above must outlive the asynchronous copies
   EMU_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
   return st;
-}
-
-emu_status mixed_potrs(emu_ctx *ctx, const emu_mat *L, double *X, long ldx, int nrhs) {
-  if (mixed_potrs_blocked_supports(L->nb)) return mixed_potrs_blocked(ctx, L, X, ldx, nrhs);
-  // nb > 1024: one thread per row and right-hand side
-  int nb = L->nb, NT = L->nt;
-  int thr = 256;
-  ProfScope ps(ctx, PROF_SOLVE, 2.0 * L->n * L->n * nrhs, 0.0);
-  for (int k = 0; k < NT; k++) {
-    if (k > 0) {
-      k_solve32_update<<<dim3((nb + thr - 1) / thr, nrhs), thr, 0, ctx->stream>>>(L->t64, L->t32, L->d_cls, nb, NT,
-                                                                                 k, 0, X, ldx);
-      EMU_LAUNCHED(ctx);
-    }
-    k_solve32_diag<<<nrhs, 512, nb * sizeof(float), ctx->stream>>>(L->t64, nb, NT, k, 0, X, ldx);
-    EMU_LAUNCHED(ctx);
-  }
-  for (int k = NT - 1; k >= 0; k--) {
-    if (k < NT - 1) {
-      k_solve32_update<<<dim3((nb + thr - 1) / thr, nrhs), thr, 0, ctx->stream>>>(L->t64, L->t32, L->d_cls, nb, NT,
-                                                                                 k, 1, X, ldx);
-      EMU_LAUNCHED(ctx);
-    }
-    k_solve32_diag<<<nrhs, 512, nb * sizeof(float), ctx->stream>>>(L->t64, nb, NT, k, 1, X, ldx);
-    EMU_LAUNCHED(ctx);
-  }
-  return EMU_OK;
 }
 
 void mixed_ctx_release(emu_ctx *ctx) {

@@ -7,10 +7,8 @@ emu_status factor_mixed(emu_ctx *ctx, emu_mat *A, const emu_mp_opts *o);
 void mixed_fill_info(const emu_mat *A, emu_factor_info *info);
 emu_status mixed_sample(emu_ctx *ctx, const emu_mat *L, const double *Z, long ldz, int s,
                         double *Y, long ldy);
-emu_status mixed_potrs(emu_ctx *ctx, const emu_mat *L, double *X, long ldx, int nrhs);
-// blocked right-looking sweeps (solve.cu), for nb a multiple of 64 up to 1024
-bool mixed_potrs_blocked_supports(int nb);
-emu_status mixed_potrs_blocked(emu_ctx *ctx, const emu_mat *L, double *X, long ldx, int nrhs);
+// X (npad x nrhs, padded rows zero) <- (L L^T)^{-1} X, L a plain or mixed factor (solve.cu)
+emu_status factor_potrs(emu_ctx *ctx, const emu_mat *L, double *X, long ldx, int nrhs);
 void mixed_ctx_release(emu_ctx *ctx);
 // graph replay and reserved-SM tuning of the single-matrix factor
 void mixed_set_schedule(emu_ctx *ctx, int use_graphs, int tuning);

@@ -4,68 +4,98 @@
 // backward error ||r||_2 / (||S||_F ||x||_2 + ||b||_2) of every column is <= tol.
 #include <math.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "mixed.h"
 
 namespace {
 
-// R[:, c0:c0+P] = B - S X for S symmetric from its packed lower FP64 tiles,
-// FP64 on the SIMT pipes: one CTA per (64-row slab of the padded matrix,
-// group of P right-hand sides), a loop over every tile column j of the slab's
-// block row i (tile (i, j) for j <= i, tile (j, i) read transposed for
-// j > i), operands staged through shared memory in 32-wide K chunks so that
-// every global read is coalesced.  Deterministic: one CTA owns each output.
+// Partial sums of S X for S symmetric from its packed lower FP64 tiles, FP64 on
+// the SIMT pipes: one CTA per (64-row slab of the padded matrix, range of tile
+// columns, group of P right-hand sides), a loop over its tile columns j (tile
+// (i, j) for j <= i, tile (j, i) read transposed for j > i), operands staged
+// through shared memory in 32-wide K chunks so that every global read is
+// coalesced.  part[z][row][P] of range z and group blockIdx.z; deterministic:
+// one CTA owns each partial sum, k_symm_finish adds the ranges in order.
+// P follows the right-hand sides (one of them cost sixteen columns' FP64 work),
+// and the ranges fill the chip where n / 64 slabs do not (60 CTAs at n = 3840).
 constexpr int RS = 64, RK = 32;
 template <int P>
 __global__ void __launch_bounds__(256)
-    k_symm_res(const double *__restrict__ t64, int nb, int NT, const double *__restrict__ X,
-               const double *__restrict__ Bm, double *__restrict__ R, long ld, int nrhs) {
-  constexpr int NQ = P / 4;  // right-hand sides per thread
+    k_symm_part(const double *__restrict__ t64, int nb, int NT, const double *__restrict__ X, double *__restrict__ part,
+                long npad, int nrhs) {
+  constexpr int KG = P == 1 ? 4 : 1;       // thread groups that share the K chunk
+  constexpr int NQ = P == 1 ? 1 : P / 4;   // right-hand sides per thread
   __shared__ double a[RK][RS + 1];
   __shared__ double x[RK][P + 1];
   const long g0 = (long)blockIdx.x * RS;
   const int i = (int)(g0 / nb), m0 = (int)(g0 % nb);
-  const int c0 = blockIdx.y * P;
+  const int c0 = blockIdx.z * P;
   const int p = min(P, nrhs - c0);
   const int tid = threadIdx.x, mm = tid & (RS - 1), q0 = tid >> 6;
+  const int j0 = (int)((long)NT * blockIdx.y / gridDim.y), j1 = (int)((long)NT * (blockIdx.y + 1) / gridDim.y);
   double acc[NQ];
 #pragma unroll
   for (int w = 0; w < NQ; w++) acc[w] = 0.0;
-  for (int j = 0; j < NT; j++) {
+  for (int j = j0; j < j1; j++) {
     const bool lower = j <= i;
     const double *T = t64 + (size_t)(lower ? tile_index(i, j, NT) : tile_index(j, i, NT)) * nb * nb;
     for (int k0 = 0; k0 < nb; k0 += RK) {
-      for (int e = tid; e < RK * RS; e += 256) {
-        if (lower) {
-          const int m = e % RS, k = e / RS;
-          a[k][m] = T[(size_t)(m0 + m) + (size_t)(k0 + k) * nb];
-        } else {
-          const int k = e % RK, m = e / RK;
-          a[k][m] = T[(size_t)(k0 + k) + (size_t)(m0 + m) * nb];
-        }
+      double v[RK * RS / 256];
+#pragma unroll
+      for (int u = 0; u < RK * RS / 256; u++) {
+        const int e = tid + 256 * u;
+        v[u] = lower ? __ldg(T + (size_t)(m0 + e % RS) + (size_t)(k0 + e / RS) * nb)
+                     : __ldg(T + (size_t)(k0 + e % RK) + (size_t)(m0 + e / RK) * nb);
+      }
+#pragma unroll
+      for (int u = 0; u < RK * RS / 256; u++) {
+        const int e = tid + 256 * u;
+        if (lower) a[e / RS][e % RS] = v[u];
+        else a[e % RK][e / RK] = v[u];
       }
       for (int e = tid; e < RK * P; e += 256) {
         const int k = e % RK, q = e / RK;
-        x[k][q] = q < p ? X[(size_t)j * nb + k0 + k + (size_t)(c0 + q) * ld] : 0.0;
+        x[k][q] = q < p ? X[(size_t)j * nb + k0 + k + (size_t)(c0 + q) * npad] : 0.0;
       }
       __syncthreads();
-#pragma unroll 4
-      for (int k = 0; k < RK; k++) {
-        const double av = a[k][mm];
+      if (KG == 4) {
 #pragma unroll
-        for (int w = 0; w < NQ; w++) acc[w] = fma(av, x[k][q0 + 4 * w], acc[w]);
+        for (int k = 0; k < RK / 4; k++) acc[0] = fma(a[k + q0 * (RK / 4)][mm], x[k + q0 * (RK / 4)][0], acc[0]);
+      } else {
+#pragma unroll 4
+        for (int k = 0; k < RK; k++) {
+          const double av = a[k][mm];
+#pragma unroll
+          for (int w = 0; w < NQ; w++) acc[w] = fma(av, x[k][q0 + 4 * w], acc[w]);
+        }
       }
       __syncthreads();
     }
   }
+  double *o = part + (((size_t)blockIdx.z * gridDim.y + blockIdx.y) * npad + g0 + mm) * P;
+  if (KG == 4) {
+    double *red = &a[0][0];
+    red[tid] = acc[0];
+    __syncthreads();
+    if (tid < RS) o[0] = (red[tid] + red[tid + 64]) + (red[tid + 128] + red[tid + 192]);
+  } else {
 #pragma unroll
-  for (int w = 0; w < NQ; w++) {
-    const int q = q0 + 4 * w;
-    if (q < p) {
-      const size_t o = (size_t)(g0 + mm) + (size_t)(c0 + q) * ld;
-      R[o] = Bm[o] - acc[w];
-    }
+    for (int w = 0; w < NQ; w++) o[q0 + 4 * w] = acc[w];
+  }
+}
+
+// R = B - the sum of the partial products' `nz` ranges, in order.
+__global__ void k_symm_finish(const double *__restrict__ part, int nz, int P, const double *__restrict__ Bm,
+                              double *__restrict__ R, long npad, int nrhs) {
+  const long total = npad * nrhs;
+  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total; e += (long)gridDim.x * blockDim.x) {
+    const long r = e % npad;
+    const int c = (int)(e / npad);
+    double s = 0.0;
+    for (int z = 0; z < nz; z++) s += part[(((size_t)(c / P) * nz + z) * npad + r) * P + c % P];
+    R[e] = Bm[e] - s;
   }
 }
 
@@ -113,9 +143,35 @@ __global__ void k_axpy(double *__restrict__ X, const double *__restrict__ D, lon
 
 }  // namespace
 
-static emu_status solve_with_factor(emu_ctx *ctx, const emu_mat *L, double *X, long ld, int nrhs) {
-  if (L->state == MAT_FACTOR64) return launch_potrs64(ctx, L, X, ld, nrhs);
-  return mixed_potrs(ctx, L, X, ld, nrhs);
+// Right-hand sides per group, groups and column ranges of the product.
+struct SymmShape {
+  int P, groups, nz;
+};
+static SymmShape symm_shape(const emu_ctx *ctx, const emu_mat *S, int nrhs) {
+  SymmShape s;
+  s.P = nrhs == 1 ? 1 : nrhs <= 4 ? 4 : nrhs <= 8 ? 8 : nrhs <= 16 ? 16 : 32;
+  s.groups = (nrhs + s.P - 1) / s.P;
+  const int slabs = S->nt * (S->nb / RS) * s.groups;
+  s.nz = std::max(1, std::min(S->nt, (6 * ctx->sm_count + slabs - 1) / slabs));
+  return s;
+}
+// R = B - S X (npad x nrhs each); part: groups nz npad P doubles.
+static emu_status symm_residual(emu_ctx *ctx, const emu_mat *S, const double *X, const double *Bp, double *R,
+                                double *part, int nrhs) {
+  const long npad = (long)S->nt * S->nb;
+  const SymmShape sh = symm_shape(ctx, S, nrhs);
+  ProfScope ps(ctx, PROF_SOLVE, 2.0 * (double)npad * npad * nrhs, 8.0 * (double)npad * npad);
+  const dim3 grid((unsigned)(npad / RS), (unsigned)sh.nz, (unsigned)sh.groups);
+  auto kern = sh.P == 1    ? k_symm_part<1>
+              : sh.P == 4  ? k_symm_part<4>
+              : sh.P == 8  ? k_symm_part<8>
+              : sh.P == 16 ? k_symm_part<16>
+                           : k_symm_part<32>;
+  kern<<<grid, 256, 0, ctx->stream>>>(S->t64, S->nb, S->nt, X, part, npad, nrhs);
+  EMU_LAUNCHED(ctx);
+  k_symm_finish<<<4 * ctx->sm_count, 256, 0, ctx->stream>>>(part, sh.nz, sh.P, Bp, R, npad, nrhs);
+  EMU_LAUNCHED(ctx);
+  return EMU_OK;
 }
 
 emu_status refine_solve(emu_ctx *ctx, const emu_mat *L, const emu_mat *S, const double *dB,
@@ -123,11 +179,12 @@ emu_status refine_solve(emu_ctx *ctx, const emu_mat *L, const emu_mat *S, const 
                         emu_refine_info *info) {
   if (nrhs == 0) return EMU_OK;
   EMU_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
-  int NT = L->nt, nb = L->nb;
-  long npad = (long)NT * nb;
+  long npad = (long)L->nt * L->nb;
   size_t blk = (size_t)npad * nrhs;
   double *buf = nullptr, *norms = nullptr;
-  EMU_CUDA_TRY(ctx, cudaMallocAsync(&buf, 4 * blk * sizeof(double), ctx->stream));
+  const SymmShape sh = symm_shape(ctx, S, nrhs);
+  const size_t part = (size_t)sh.groups * sh.nz * npad * sh.P;
+  EMU_CUDA_TRY(ctx, cudaMallocAsync(&buf, (4 * blk + part) * sizeof(double), ctx->stream));
   EMU_CUDA_TRY(ctx, cudaMallocAsync(&norms, 3 * nrhs * sizeof(double), ctx->stream));
   double *Bp = buf, *X = buf + blk, *R = buf + 2 * blk, *D = buf + 3 * blk;
   std::vector<double> hn(3 * nrhs);
@@ -146,19 +203,10 @@ emu_status refine_solve(emu_ctx *ctx, const emu_mat *L, const emu_mat *S, const 
   // X0 = M^{-1} B
   if (s == EMU_OK) {
     e = cudaMemcpyAsync(X, Bp, blk * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream);
-    s = (e == cudaSuccess) ? solve_with_factor(ctx, L, X, npad, nrhs) : emu_cuda_fail(ctx, e, "refine x0");
+    s = (e == cudaSuccess) ? factor_potrs(ctx, L, X, npad, nrhs) : emu_cuda_fail(ctx, e, "refine x0");
   }
   while (s == EMU_OK) {
-    {
-      ProfScope ps(ctx, PROF_SOLVE, 2.0 * (double)npad * npad * nrhs, 8.0 * (double)npad * npad);
-      if (nrhs <= 16)
-        k_symm_res<16><<<dim3((unsigned)(npad / RS), 1), 256, 0, ctx->stream>>>(S->t64, nb, NT, X, Bp, R, npad,
-                                                                                nrhs);
-      else
-        k_symm_res<32><<<dim3((unsigned)(npad / RS), (nrhs + 31) / 32), 256, 0, ctx->stream>>>(S->t64, nb, NT, X,
-                                                                                              Bp, R, npad, nrhs);
-    }
-    ctx->launches++;
+    if ((s = symm_residual(ctx, S, X, Bp, R, buf + 4 * blk, nrhs)) != EMU_OK) break;
     k_col_norms<<<nrhs, 256, 0, ctx->stream>>>(R, X, Bp, npad, npad, norms);
     ctx->launches++;
     e = cudaGetLastError();
@@ -185,7 +233,7 @@ emu_status refine_solve(emu_ctx *ctx, const emu_mat *L, const emu_mat *S, const 
       s = emu_cuda_fail(ctx, e, "refine copy");
       break;
     }
-    s = solve_with_factor(ctx, L, D, npad, nrhs);
+    s = factor_potrs(ctx, L, D, npad, nrhs);
     if (s != EMU_OK) break;
     k_axpy<<<4 * ctx->sm_count, 256, 0, ctx->stream>>>(X, D, (long)blk);
     ctx->launches++;
