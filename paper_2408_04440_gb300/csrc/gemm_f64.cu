@@ -62,70 +62,6 @@ struct Shared {
 };
 static_assert(sizeof(Shared) <= BAR_BYTES, "barrier block");
 
-// Adds the chunk's sum_g G_g 2^-7(g+2), for the group sums G_g of one output
-// (column x of r[g]), to the exact fixed-point accumulator (hi, lo) of value
-// hi 2^-31 + lo 2^-63 (lo unsigned, below 2^32).  Each G_g is an integer held
-// exactly in FP32 (below 2^24, see the header), so the chunk's sum is formed
-// in integer arithmetic: groups 2..7 by Horner in 64 bits, T = sum_{g>=2}
-// G_g 2^(7(7-g)), |T| < 2^59 (|G_g| < 2^24 for g >= 1 with KCHUNK = 384:
-// at most two products of a leading digit, |d_0| <= 128, and g - 1 of
-// trailing digits, |d_p| <= 64, per K term), and groups 0..1 as Q = 2^7 G_0
-// + G_1, |Q| < 2^30 (|G_0| <= 384 * 2^14, |G_1| <= 384 * 2^14).  The chunk's value is Q 2^-21 + T 2^-63
-// = (2^10 Q + floor(T / 2^32)) 2^-31 + (T mod 2^32) 2^-63; the low word's
-// carry moves into hi, which grows by less than 2^41 per chunk.  No FP64
-// instruction runs per chunk: the FP64 pipe, GB300's slowest unit, is used for
-// one add per output at the end of the item.
-static_assert(NS == 8 && SLICE_BITS == 7 && KCHUNK <= 384, "fold_groups is written for 8 digits of 7 bits");
-__device__ __forceinline__ void fold_groups(const uint32_t (&r)[NS][2], int x, long long &hi, unsigned &lo) {
-  int gi[NS];
-#pragma unroll
-  for (int g = 0; g < NS; g++) gi[g] = __float2int_rn(__uint_as_float(r[g][x]));  // exact: integers below 2^24
-  long long t = gi[2];
-#pragma unroll
-  for (int g = 3; g < NS; g++) t = t * 128 + gi[g];
-  const long long q = gi[0] * 128 + gi[1];
-  const unsigned l = lo + (unsigned)t;  // low 32 bits of T, modulo 2^32
-  hi += q * 1024 + (t >> 32) + (l < lo ? 1 : 0);  // arithmetic shift: floor; carry of the low word
-  lo = l;
-}
-// (hi 2^-31 + lo 2^-63) 2^s rounded once to FP64 (ties to even), for s that
-// keeps the result in the normal range: normalised, rounded and packed in
-// integer arithmetic.  Two conversions, an FMA and a multiply on the FP64 pipe
-// took about 20 k cycles per 128 x 64 block, as long as the MMAs of K = 256.
-// s out of range: the same value through FP64 arithmetic (fixed_scaled_any).
-__device__ double fixed_scaled_any(long long hi, unsigned lo, int s);
-__device__ __forceinline__ double fixed_scaled(long long hi, unsigned lo, int s) {
-  const bool neg = hi < 0;
-  // |hi 2^32 + lo| = ahi 2^32 + alo
-  const unsigned alo = neg ? 0u - lo : lo;
-  const unsigned long long ahi = (unsigned long long)(neg ? ~hi + (lo == 0u) : hi);
-  unsigned long long t;  // the leading 64 bits, top bit set
-  int lz;
-  bool sticky = false;
-  if (ahi != 0) {
-    lz = __clzll((long long)ahi);
-    t = ahi << lz;
-    if (lz >= 32) {
-      t |= (unsigned long long)alo << (lz - 32);
-    } else {
-      t |= (unsigned long long)alo >> (32 - lz);
-      sticky = (alo << lz) != 0u;
-    }
-  } else {
-    if (alo == 0u) return s > kExpPoison / 2 ? fixed_scaled_any(hi, lo, s) : 0.0;  // a poisoned row's digits are 0
-    const int l = __clz((int)alo);
-    t = (unsigned long long)alo << (32 + l);
-    lz = 64 + l;
-  }
-  const int e = 1055 - lz + s;  // biased exponent
-  if (e < 1 || e > 2045) return fixed_scaled_any(hi, lo, s);
-  unsigned long long m = t >> 11;
-  const unsigned rem = (unsigned)t & 0x7ffu;
-  m += (rem > 0x400u || (rem == 0x400u && (sticky || (m & 1ull)))) ? 1ull : 0ull;
-  m += (unsigned long long)(e - 1) << 52;  // the implicit bit adds one to the exponent; so does a carry
-  return __longlong_as_double((long long)(m | (neg ? 0x8000000000000000ull : 0ull)));
-}
-
 __device__ inline bool failed(const int *st) { return *((volatile const int *)st) != DEV_OK; }
 
 __device__ inline void raise_timeout(Shared *sh, int *status) {
@@ -134,16 +70,6 @@ __device__ inline void raise_timeout(Shared *sh, int *status) {
 }
 
 // ------------------------------------------------------------- digits
-// 2^e for integer e in the normal range (exact).
-__device__ inline double exp2i(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
-// fixed_scaled for any s: near the ends of the FP64 range, and NaN where s
-// carries the poison of a row with an infinity or a NaN.
-__device__ __noinline__ double fixed_scaled_any(long long hi, unsigned lo, int s) {
-  if (s > kExpPoison / 2) return __longlong_as_double(0x7ff8000000000000ll);
-  const double x = fma((double)hi, 0x1p-31, (double)lo * 0x1p-63);
-  const int s1 = max(-1000, min(1000, s));
-  return x * exp2i(s1) * exp2i(max(-1000, min(1000, s - s1)));
-}
 // A 32 x 32 block (256 threads) in shared memory, row rr with exponent
 // exp(rr), to its digit planes at d + rr * ld: a half warp per row, two
 // columns per lane.

@@ -52,14 +52,11 @@ def test_fixed_point_words_and_digits(kind):
         e = max(e0 + rng.choice((0, 0, 1, 20, 54, 55, 56, 57, 58, 100)), -960)
         X = _to_fixed(x, e)
         assert abs(X) == _round_even(abs(Fraction(x)) * Fraction(2) ** (56 - e)) <= 2**56
-        back = 0
-        for p in range(8):
-            sh = 7 * (7 - p)
-            d = (X + (1 << (sh - 1))) >> sh if sh else X
-            X -= d << sh
-            assert abs(d) <= (128 if p == 0 else 64)
-            back += d << sh
-        assert X == 0 and back == _to_fixed(x, e)
+        # the digits as the fields of X with 64 added at every digit but the first
+        Y = X + sum(64 << (7 * q) for q in range(7))
+        digits = [Y >> 49] + [((Y >> (7 * (7 - p))) & 127) - 64 for p in range(1, 8)]
+        assert abs(digits[0]) <= 128 and all(abs(d) <= 64 for d in digits[1:])
+        assert sum(d << (7 * (7 - p)) for p, d in enumerate(digits)) == X
 
 
 def _fixed_scaled(hi, lo, s):

@@ -59,3 +59,30 @@ def test_refined_solves(E, ctx, L, nb, r, eps):
     assert _backward(O.cov_build(L, 4.0), X.cpu().numpy(), B.cpu().numpy()) <= 1e-14 + 2 * L * L * 2.0**-53
     again, _ = E.emu_solve_refine(ctx, A, S, B, tol=1e-14)
     assert (again == X).all()
+
+
+@pytest.mark.parametrize("L,nb,r", [(46, 128, 2), (46, 256, 16), (46, 512, 17), (47, 384, 33)])
+def test_residuals_as_digit_products(E, ctx, L, nb, r):
+    """From 2048 rows on: chunks of 128 and 256, ragged tiles, groups of 16; a matrix whose rows are scaled by powers of
+    two over 2^-40 .. 2^40 converges as it does unscaled, and one that is not positive semidefinite is solved too."""
+    import torch
+
+    n = L * L
+    S0 = O.cov_build(L, 4.0)
+    d = 2.0 ** np.random.default_rng(L).integers(-20, 21, n)
+    for kind in ("plain", "scaled", "indefinite"):
+        M = S0 * d[:, None] * d[None, :] if kind == "scaled" else S0.copy()
+        A = E.emu_mat_import(ctx, torch.from_numpy(M).cuda(), nb)
+        E.emu_potrf_mp(ctx, A)
+        if kind == "indefinite":  # refine against another matrix: one entry above its rows' diagonals
+            M[1500, 1400] = M[1400, 1500] = 1e-5
+        S = E.emu_mat_import(ctx, torch.from_numpy(M).cuda(), nb)
+        B = _rhs(n, r)
+        X, info = E.emu_solve_refine(ctx, A, S, B, tol=1e-14, raise_on_error=False)
+        X, Bn = X.cpu().numpy(), B.cpu().numpy()
+        if kind != "indefinite":
+            assert info.status == E.EMU_OK
+        # the residual the call reports is the one its iterate has
+        have = np.max(np.linalg.norm(Bn - M @ X, axis=0)
+                      / (np.linalg.norm(M) * np.linalg.norm(X, axis=0) + np.linalg.norm(Bn, axis=0)))
+        assert abs(have - info.rel_resid) <= 1e-6 * have + 2 * n * 2.0**-53
