@@ -12,6 +12,7 @@
 
 #include <algorithm>
 
+#include "convert.cuh"
 #include "emu_internal.h"
 
 namespace {
@@ -455,7 +456,7 @@ __device__ inline void export_chunk(int n, int nb, int NT, int ti, int tj, int c
       if (gi >= n) break;
       double v = 0.0;
       if (gi >= gj) {
-        if (tile32) v = (double)tile32[r + (size_t)c * nb];
+        if (tile32) v = f64_of(tile32[r + (size_t)c * nb]);
         else if (tile) v = tile[r + (size_t)c * nb];
       }
       out[gi + gj * ld] = v;

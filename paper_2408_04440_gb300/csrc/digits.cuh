@@ -44,13 +44,24 @@ __device__ inline long long to_fixed(double x, int e) {
   return (long long)b < 0 ? -(long long)X : (long long)X;
 }
 
-// The NS digits of X (|X| <= 2^56, the unit of the last digit is 2^-56):
-// |digit 0| <= 128, -64 <= digit p < 64 for p >= 1 and
-// sum_p digit_p 2^(7 (NS - 1 - p)) = X exactly.  With 64 added at every digit
-// but the first, the biased digits are the 7-bit fields of X.  As BF16 bits: a
-// digit is at most eight bits wide, so the upper half of its FP32 pattern
-// (formed by an add to 2^23, no conversion) is exact.
+// The NS digits of X (|X| <= 2^56, the unit of the last digit is 2^-56): peeled
+// off from the top, each rounded to nearest, so |digit 0| <= 128 and
+// |digit p| <= 64 for p >= 1 and sum_p digit_p 2^(7 (NS - 1 - p)) = X exactly.
+// As BF16 bits: a digit is at most eight bits wide, so the upper half of its
+// FP32 pattern (formed by an add of 1.5 2^23, no conversion) is exact.
 __device__ inline void digit_bits(long long X, uint32_t (&d)[NS]) {
+#pragma unroll
+  for (int p = 0; p < NS; p++) {
+    const int sh = SLICE_BITS * (NS - 1 - p);
+    const long long dg = (sh > 0) ? ((X + (1LL << (sh > 0 ? sh - 1 : 0))) >> sh) : X;
+    X -= dg << sh;
+    d[p] = __float_as_uint(__int_as_float(0x4B400000 + (int)dg) - 12582912.0f) >> 16;
+  }
+}
+// Digits with the same bounds and sum (-64 <= digit p < 64 for p >= 1) at a
+// third of the instructions: with 64 added at every digit but the first, the
+// biased digits are the 7-bit fields of X.
+__device__ inline void field_digit_bits(long long X, uint32_t (&d)[NS]) {
   constexpr long long kBias = 0x1020408102040LL;  // sum of 64 2^(7 q), q = 0 .. NS - 2
   const long long Y = X + kBias;
   const int top = (int)(Y >> (SLICE_BITS * (NS - 1)));

@@ -25,6 +25,7 @@
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 
+#include "convert.cuh"
 #include "gemm_tc.h"
 #include "tc.cuh"
 
@@ -306,7 +307,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             for (int x = 0; x < 32; x++) c[x] = (x < nval) ? __ldcg(o + (long)x * ldo) : 0.0;
 #pragma unroll
             for (int x = 0; x < 32; x++)
-              if (x < nval) __stcg(o + (long)x * ldo, c[x] + (double)__uint_as_float(r[x]));
+              if (x < nval) __stcg(o + (long)x * ldo, c[x] + f64_of(__uint_as_float(r[x])));
           }
         }
       }

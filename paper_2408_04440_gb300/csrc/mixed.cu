@@ -19,6 +19,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "convert.cuh"
 #include "gemm_f64.h"
 #include "gemm_tc.h"
 #include "mixed.h"
@@ -41,14 +42,10 @@ __device__ inline void split3(float x, uint16_t &p0, uint16_t &p1, uint16_t &p2)
   p2 = __bfloat16_as_ushort(b2);
 }
 __device__ inline void split3(double x, uint16_t &p0, uint16_t &p1, uint16_t &p2) {
-  __nv_bfloat16 b0 = __double2bfloat16(x);
-  double r1 = x - (double)__bfloat162float(b0);
-  __nv_bfloat16 b1 = __double2bfloat16(r1);
-  double r2 = r1 - (double)__bfloat162float(b1);
-  __nv_bfloat16 b2 = __double2bfloat16(r2);
-  p0 = __bfloat16_as_ushort(b0);
-  p1 = __bfloat16_as_ushort(b1);
-  p2 = __bfloat16_as_ushort(b2);
+  p0 = bf16_of(x);
+  const double r1 = x - f64_of_bf16(p0);
+  p1 = bf16_of(r1);
+  p2 = bf16_of(r1 - f64_of_bf16(p1));
 }
 
 // FP32 masters of the low-precision tiles: t32 = (float) t64.
@@ -56,11 +53,12 @@ __global__ void k_to_f32(const double *__restrict__ t64, float *__restrict__ t32
                          const unsigned char *__restrict__ cls, size_t tile_elems) {
   long t = blockIdx.y;
   if (cls[t] == EMU_CLASS_FP64) return;
-  const double *s = t64 + (size_t)t * tile_elems;
-  float *d = t32 + (size_t)t * tile_elems;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < tile_elems;
-       e += (size_t)gridDim.x * blockDim.x)
-    d[e] = (float)s[e];
+  const double2 *s = reinterpret_cast<const double2 *>(t64 + (size_t)t * tile_elems);
+  float4 *d = reinterpret_cast<float4 *>(t32 + (size_t)t * tile_elems);
+  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < tile_elems / 4; e += (size_t)gridDim.x * blockDim.x) {
+    const double2 v = s[2 * e], w = s[2 * e + 1];
+    d[e] = make_float4(f32_of(v.x), f32_of(v.y), f32_of(w.x), f32_of(w.y));
+  }
 }
 
 // Widen one FP32 master tile into the FP64 arena (before its POTRF).
@@ -69,7 +67,7 @@ __global__ void k_tile_to_f64(const float *__restrict__ s, double *__restrict__ 
   if (failed(st)) return;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < tile_elems;
        e += (size_t)gridDim.x * blockDim.x)
-    d[e] = (double)s[e];
+    d[e] = f64_of(s[e]);
 }
 
 // FP32 copy of the FP64 diagonal factor tile L_kk for the FP32 panel TRSM
@@ -79,7 +77,7 @@ __global__ void k_diag_to_f32(const double *__restrict__ s, float *__restrict__ 
   if (failed(st)) return;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < tile_elems;
        e += (size_t)gridDim.x * blockDim.x)
-    d[e] = (float)s[e];
+    d[e] = f32_of(s[e]);
 }
 
 // Three BF16 pieces, row-major, of whole tiles from their FP64 (or FP32)
@@ -196,13 +194,16 @@ __global__ void __launch_bounds__(1024)
 // TRSM's 128-row block, or nb - 64 > 512 TMEM columns): L_ik = A_ik L_kk^{-T} from the FP32 master A_ik and an FP32 copy
 // of the FP64 L_kk, written back to the master and, split, to the operand
 // arena.
-// One CTA per (row block, tile); warp w owns rows w + NW*q, a lane owns one
-// column of the current 32-column block cb.  L_kk streams through shared
-// memory as 32x32 chunks (rows of block cb, columns of block c <= cb) in a
-// ring of NBUF buffers filled by cp.async several chunks ahead, the same
-// sequence for every CTA: a chunk c < cb is subtracted from the block's
-// columns (four independent partial sums per row), the diagonal chunk c = cb
-// is solved by forward substitution with shuffles.  One barrier per chunk.
+// One CTA of four warps per (ROWS rows, tile), lane = column of the current
+// 32-column block cb.  L_kk streams through shared memory as 32x32 chunks (rows
+// of block cb, columns of block c <= cb) in a ring of NBUF buffers filled by
+// cp.async several chunks ahead, the same sequence for every CTA.  An entry is
+// the sum of four partial sums over the columns p = w mod 4: warp w forms its
+// one for all rows of the CTA, so that a value of L_kk read from shared memory
+// serves ROWS FMAs and a 16-byte read of X four (X is stored by p mod 4); the
+// warps then exchange the sums and solve the diagonal chunk by forward
+// substitution with shuffles, ROWS / 4 rows each.  (With the four sums of two
+// rows in one warp every FMA waited for its own read of L_kk.)
 constexpr int TS_LD_PAD = 4;
 constexpr int TS_CHUNK = B * B;  // floats per chunk, column-major (32 columns x 32 rows)
 constexpr int TS_NBUF_CRIT = 8;   // chunk buffers, single critical-path tile (1 CTA per SM)
@@ -218,21 +219,23 @@ __device__ inline void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// NW warps, RPW rows per warp, NBUF chunk buffers: 16-row CTAs (8 warps x 2)
-// for throughput on the panel, 4-row CTAs (4 warps x 1, deeper ring) for the
-// single tile on the critical path, where more CTAs in parallel mean less
-// latency.
-template <int NW, int RPW, int NBUF, bool JOBS = false>
-__global__ void __launch_bounds__(NW * 32)
+// Column c of X's 32-column blocks: the eight columns of a partial sum together.
+__device__ inline int ts_perm(int c) { return (c & ~31) | ((c & 3) << 3) | ((c & 31) >> 2); }
+
+// 16-row CTAs for throughput on the panel; 8-row CTAs with a deeper ring for
+// the single tile on the critical path, where more CTAs mean less latency.
+template <int ROWS, int NBUF, bool JOBS = false>
+__global__ void __launch_bounds__(128)
     k_trsm32_panel(const float *__restrict__ Lkk0, float *__restrict__ t32, uint16_t *__restrict__ op, int nb,
                    int NT, int k, const int *__restrict__ rows, const int *st,
                    const int2 *__restrict__ jobs = nullptr) {
-  constexpr int ROWS = NW * RPW, NTH = NW * 32;
+  constexpr int NTH = 128, RW = ROWS / 4;
   if (failed(st)) return;
   extern __shared__ __align__(16) float sm[];
   const int ldx = nb + TS_LD_PAD;
   float *S = sm;                     // [NBUF][32][32]: chunk ring, S[p * 32 + r] = L_kk(cb*32 + r, c*32 + p)
   float *X = sm + NBUF * TS_CHUNK;   // [ROWS][ldx]: the CTA's rows of A_ik, solved in place
+  float *E = X + ROWS * ldx;         // [4][ROWS][32]: partial sums
   int r0 = blockIdx.x * ROWS;
   // tile (i, k) of one matrix, or (batched) an explicit tile index and the
   // slot of its L_kk copy
@@ -270,78 +273,77 @@ __global__ void __launch_bounds__(NW * 32)
 #pragma unroll 8
   for (int e = tid; e < ROWS * nb; e += NTH) {
     int r = e % ROWS, c = e / ROWS;
-    X[r * ldx + c] = A[r + (size_t)c * nb];
+    X[r * ldx + ts_perm(c)] = A[r + (size_t)c * nb];
   }
+  __syncthreads();
   int i = 0;
   for (int cb = 0; cb < nbc; cb++) {
-    float a0[RPW], a1[RPW], a2[RPW], a3[RPW];
-    for (int c = 0; c <= cb; c++, i++) {
+    float a[ROWS];
+#pragma unroll
+    for (int q = 0; q < ROWS; q++) a[q] = w == 0 ? X[q * ldx + cb * B + ts_perm(lane)] : 0.f;
+    for (int c = 0; c < cb; c++, i++) {
       cp_async_wait<NBUF - 2>();  // this thread's copies of chunk i have landed
       __syncthreads();            // everyone's; and chunk i-1's buffer is free
       issue();
       const float *Sc = S + (i % NBUF) * TS_CHUNK;
-      if (c == 0) {
+      float l[8];
 #pragma unroll
-        for (int q = 0; q < RPW; q++) {
-          a0[q] = X[(w + NW * q) * ldx + cb * B + lane];
-          a1[q] = a2[q] = a3[q] = 0.f;
+      for (int u = 0; u < 8; u++) l[u] = Sc[(4 * u + w) * B + lane];
+      const float *Xc = X + c * B + w * 8;
+#pragma unroll
+      for (int h = 0; h < 2; h++)
+#pragma unroll
+        for (int q = 0; q < ROWS; q++) {
+          const float4 xv = *reinterpret_cast<const float4 *>(Xc + q * ldx + 4 * h);
+          a[q] = fmaf(-xv.x, l[4 * h], a[q]);
+          a[q] = fmaf(-xv.y, l[4 * h + 1], a[q]);
+          a[q] = fmaf(-xv.z, l[4 * h + 2], a[q]);
+          a[q] = fmaf(-xv.w, l[4 * h + 3], a[q]);
         }
-      }
-      if (c < cb) {
+    }
+    // diagonal chunk
 #pragma unroll
-        for (int q = 0; q < RPW; q++) {
-          const float4 *xq = reinterpret_cast<const float4 *>(X + (w + NW * q) * ldx + c * B);
+    for (int q = 0; q < ROWS; q++) E[(w * ROWS + q) * B + lane] = a[q];
+    cp_async_wait<NBUF - 2>();
+    __syncthreads();
+    issue();
+    const float *Sc = S + (i % NBUF) * TS_CHUNK;
+    i++;
+    const float myrinv = 1.0f / Sc[lane * B + lane];
+    float v[RW];
 #pragma unroll
-          for (int p4 = 0; p4 < B / 4; p4++) {
-            const float4 xv = xq[p4];
-            a0[q] -= xv.x * Sc[(4 * p4 + 0) * B + lane];
-            a1[q] -= xv.y * Sc[(4 * p4 + 1) * B + lane];
-            a2[q] -= xv.z * Sc[(4 * p4 + 2) * B + lane];
-            a3[q] -= xv.w * Sc[(4 * p4 + 3) * B + lane];
-          }
-        }
-      } else {
-        // diagonal chunk: ld[p] = L_kk(cb*32 + lane, cb*32 + p) for p <= lane
-        float ld[B];
+    for (int u = 0; u < RW; u++) {
+      const float *e = E + (w * RW + u) * B + lane;
+      v[u] = (e[0] + e[ROWS * B]) + (e[2 * ROWS * B] + e[3 * ROWS * B]);
+    }
+#pragma unroll 8
+    for (int j = 0; j < B; j++) {
+      const float rj = __shfl_sync(0xffffffffu, myrinv, j);
+      const float lj = lane > j ? Sc[j * B + lane] : 0.f;  // L_kk(cb*32 + lane, cb*32 + j)
 #pragma unroll
-        for (int p = 0; p < B; p++) ld[p] = (p <= lane) ? Sc[p * B + lane] : 0.f;
-        float mydiag = ld[0];
-#pragma unroll
-        for (int p = 1; p < B; p++)
-          if (p == lane) mydiag = ld[p];
-        const float myrinv = 1.0f / mydiag;
-        float a[RPW];
-#pragma unroll
-        for (int q = 0; q < RPW; q++) a[q] = (a0[q] + a1[q]) + (a2[q] + a3[q]);
-#pragma unroll
-        for (int j = 0; j < B; j++) {
-          float rj = __shfl_sync(0xffffffffu, myrinv, j);
-#pragma unroll
-          for (int q = 0; q < RPW; q++) {
-            float xj = __shfl_sync(0xffffffffu, a[q], j) * rj;
-            if (lane == j) a[q] = xj;
-            if (lane > j) a[q] -= xj * ld[j];
-          }
-        }
-#pragma unroll
-        for (int q = 0; q < RPW; q++) X[(w + NW * q) * ldx + cb * B + lane] = a[q];
+      for (int u = 0; u < RW; u++) {
+        const float xj = __shfl_sync(0xffffffffu, v[u], j) * rj;
+        if (lane == j) v[u] = xj;
+        if (lane > j) v[u] = fmaf(-xj, lj, v[u]);
       }
     }
+#pragma unroll
+    for (int u = 0; u < RW; u++) X[(w * RW + u) * ldx + cb * B + ts_perm(lane)] = v[u];
+    __syncthreads();
   }
   cp_async_wait<0>();
-  __syncthreads();
   // FP32 master (column-major) and the sender-side BF16 pieces (row-major)
 #pragma unroll 8
   for (int e = tid; e < ROWS * nb; e += NTH) {
     int r = e % ROWS, c = e / ROWS;
-    A[r + (size_t)c * nb] = X[r * ldx + c];
+    A[r + (size_t)c * nb] = X[r * ldx + ts_perm(c)];
   }
   size_t plane = (size_t)nb * nb;
   uint16_t *P = op + (size_t)ti * 3 * plane + (size_t)r0 * nb;
   for (int e = tid; e < ROWS * nb; e += NTH) {
     int r = e / nb, c = e % nb;
     uint16_t p0, p1, p2;
-    split3(X[r * ldx + c], p0, p1, p2);
+    split3(X[r * ldx + ts_perm(c)], p0, p1, p2);
     size_t off = (size_t)r * nb + c;
     P[off] = p0;
     P[plane + off] = p1;
@@ -350,7 +352,7 @@ __global__ void __launch_bounds__(NW * 32)
 }
 
 static size_t trsm32_smem(int nb, int rows, int nbuf) {
-  return (size_t)(nbuf * TS_CHUNK + rows * (nb + TS_LD_PAD)) * sizeof(float);
+  return (size_t)(nbuf * TS_CHUNK + rows * (nb + TS_LD_PAD) + 4 * rows * B) * sizeof(float);
 }
 
 // z pieces for the sampler: zp[q][n][k] = piece q of Z[k][n], n < s_pad
@@ -1063,11 +1065,11 @@ static emu_status factor_mixed_record(emu_ctx *ctx, emu_mat *A, MixedPlan *P, in
   cudaEvent_t ev_start = ctx->sched_ev[EV * NT], ev_end = ctx->sched_ev[EV * NT + 1];
   EMU_CUDA_TRY(ctx, cudaEventRecord(ev_start, user));
   for (cudaStream_t q : {ctx->crit, ctx->mid, ctx->bulk}) EMU_CUDA_TRY(ctx, cudaStreamWaitEvent(q, ev_start, 0));
-  size_t tsm16 = trsm32_smem(nb, 16, TS_NBUF_PANEL), tsm4 = trsm32_smem(nb, 4, TS_NBUF_CRIT);
-  EMU_CUDA_TRY(ctx, cudaFuncSetAttribute(k_trsm32_panel<8, 2, TS_NBUF_PANEL>,
+  size_t tsm16 = trsm32_smem(nb, 16, TS_NBUF_PANEL), tsm8 = trsm32_smem(nb, 8, TS_NBUF_CRIT);
+  EMU_CUDA_TRY(ctx, cudaFuncSetAttribute(k_trsm32_panel<16, TS_NBUF_PANEL>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm16));
-  EMU_CUDA_TRY(ctx, cudaFuncSetAttribute(k_trsm32_panel<4, 1, TS_NBUF_CRIT>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm4));
+  EMU_CUDA_TRY(ctx, cudaFuncSetAttribute(k_trsm32_panel<8, TS_NBUF_CRIT>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm8));
 
   // TRSM of the listed rows of panel k: FP64 rows on the FP64 pipe, then split;
   // low-class rows on the tensor cores (trsm_tc.cu), else the SIMT kernel
@@ -1153,10 +1155,10 @@ static emu_status factor_mixed_record(emu_ctx *ctx, emu_mat *A, MixedPlan *P, in
       ProfScope ps(ctx, PROF_TRSM32, n32 * nb3, 14.0 * n32 * te);
       const float *lkk = P->d_lkk32 + (size_t)(k & 1) * te;
       if (critical)
-        k_trsm32_panel<4, 1, TS_NBUF_CRIT><<<dim3(nb / 4, n32), 128, tsm4, ctx->stream>>>(
+        k_trsm32_panel<8, TS_NBUF_CRIT><<<dim3(nb / 8, n32), 128, tsm8, ctx->stream>>>(
             lkk, A->t32, A->op_bf16, nb, NT, k, P->d_rows32 + r32, st);
       else
-        k_trsm32_panel<8, 2, TS_NBUF_PANEL><<<dim3(nb / 16, n32), 256, tsm16, ctx->stream>>>(
+        k_trsm32_panel<16, TS_NBUF_PANEL><<<dim3(nb / 16, n32), 128, tsm16, ctx->stream>>>(
             lkk, A->t32, A->op_bf16, nb, NT, k, P->d_rows32 + r32, st);
       EMU_LAUNCHED(ctx);
     }
@@ -1485,7 +1487,7 @@ __global__ void k_tiles_to_f64(const float *__restrict__ t32, double *__restrict
   if (failed(st)) return;
   size_t base = (size_t)tiles[blockIdx.y] * te;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < te; e += (size_t)gridDim.x * blockDim.x)
-    t64[base + e] = (double)t32[base + e];
+    t64[base + e] = f64_of(t32[base + e]);
 }
 
 // FP32 copies of listed FP64 diagonal factor tiles into consecutive slots.
@@ -1495,7 +1497,7 @@ __global__ void k_diag_to_f32_slots(const double *__restrict__ t64, float *__res
   size_t base = (size_t)tiles[blockIdx.y] * te;
   float *d = slots + (size_t)blockIdx.y * te;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < te; e += (size_t)gridDim.x * blockDim.x)
-    d[e] = (float)t64[base + e];
+    d[e] = f32_of(t64[base + e]);
 }
 
 }  // namespace
@@ -1512,7 +1514,7 @@ emu_status launch_to_f32_tiles(emu_ctx *ctx, const double *t64, float *t32, cons
 emu_status launch_tiles_to_f64(emu_ctx *ctx, const float *t32, double *t64, const long *d_tiles, int n, size_t te) {
   if (n <= 0) return EMU_OK;
   ProfScope ps(ctx, PROF_SPLIT, 0.0, 12.0 * n * te);
-  k_tiles_to_f64<<<dim3(16, n), 256, 0, ctx->stream>>>(t32, t64, d_tiles, te, ctx->d_status);
+  k_tiles_to_f64<<<dim3((unsigned)std::max<size_t>(16, te / 1024), n), 256, 0, ctx->stream>>>(t32, t64, d_tiles, te, ctx->d_status);
   EMU_LAUNCHED(ctx);
   return EMU_OK;
 }
@@ -1521,7 +1523,8 @@ emu_status launch_diag_to_f32_slots(emu_ctx *ctx, const double *t64, float *slot
                                     size_t te) {
   if (n <= 0) return EMU_OK;
   ProfScope ps(ctx, PROF_SPLIT, 0.0, 12.0 * n * te);
-  k_diag_to_f32_slots<<<dim3(16, n), 256, 0, ctx->stream>>>(t64, slots, d_tiles, te, ctx->d_status);
+  // a few listed tiles, on the critical stream: four entries per thread
+  k_diag_to_f32_slots<<<dim3((unsigned)std::max<size_t>(16, te / 1024), n), 256, 0, ctx->stream>>>(t64, slots, d_tiles, te, ctx->d_status);
   EMU_LAUNCHED(ctx);
   return EMU_OK;
 }
@@ -1529,13 +1532,15 @@ emu_status launch_diag_to_f32_slots(emu_ctx *ctx, const double *t64, float *slot
 emu_status launch_trsm32_jobs(emu_ctx *ctx, const float *slots, float *t32, uint16_t *op, int nb, const int2 *d_jobs,
                               int njobs) {
   if (njobs <= 0) return EMU_OK;
-  size_t sm = trsm32_smem(nb, 16, TS_NBUF_PANEL);
-  EMU_CUDA_TRY(ctx, cudaFuncSetAttribute(k_trsm32_panel<8, 2, TS_NBUF_PANEL, true>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  // the critical form where 16-row CTAs of the jobs do not fill the chip
+  const bool few = njobs * (nb / 16) < 2 * ctx->sm_count;
+  size_t sm = few ? trsm32_smem(nb, 8, TS_NBUF_CRIT) : trsm32_smem(nb, 16, TS_NBUF_PANEL);
+  auto kern = few ? k_trsm32_panel<8, TS_NBUF_CRIT, true> : k_trsm32_panel<16, TS_NBUF_PANEL, true>;
+  EMU_CUDA_TRY(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   double nb3 = (double)nb * nb * nb;
   ProfScope ps(ctx, PROF_TRSM32, njobs * nb3, 14.0 * njobs * nb * nb);
-  k_trsm32_panel<8, 2, TS_NBUF_PANEL, true><<<dim3(nb / 16, njobs), 256, sm, ctx->stream>>>(
-      slots, t32, op, nb, 0, 0, nullptr, ctx->d_status, d_jobs);
+  kern<<<dim3(nb / (few ? 8 : 16), njobs), 128, sm, ctx->stream>>>(slots, t32, op, nb, 0, 0, nullptr, ctx->d_status,
+                                                                   d_jobs);
   EMU_LAUNCHED(ctx);
   return EMU_OK;
 }

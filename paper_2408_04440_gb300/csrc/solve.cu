@@ -25,6 +25,7 @@
 // and 33 ms.
 #include <algorithm>
 
+#include "convert.cuh"
 #include "mixed.h"
 
 namespace {
@@ -37,20 +38,10 @@ constexpr long long kSweepWaitCycles = 4000000000ll;
 
 __device__ inline bool failed(const int *st) { return *((volatile const int *)st) != DEV_OK; }
 
-// FP64 -> FP32, round to nearest even, in integer arithmetic where the result
-// is a normal FP32 (a conversion holds the FP64 pipe for 19 cycles per warp).
-__device__ inline float to_f32(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int ex = (int)(b >> 52) & 0x7ff;
-  if (ex < 898 || ex > 1149) return (float)x;
-  const unsigned long long r = b + 0x0fffffffull + ((b >> 29) & 1ull);
-  const unsigned m = (unsigned)(r >> 29) - (896u << 23);  // low 31 bits: exponent and fraction
-  return __uint_as_float((m & 0x7fffffffu) | ((unsigned)(b >> 32) & 0x80000000u));
-}
 template <typename F>
 __device__ inline F from_f64(double x);
 template <>
-__device__ inline float from_f64<float>(double x) { return to_f32(x); }
+__device__ inline float from_f64<float>(double x) { return f32_of(x); }
 template <>
 __device__ inline double from_f64<double>(double x) { return x; }
 

@@ -364,8 +364,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             // |x| < 2^e, else the bound failed
             const unsigned long long m0 = gemm64::mag_bits(v[x0]), m1 = gemm64::mag_bits(v[x0 + 1]);
             bad |= (int)((m0 >> 52) & 0x7ff) - 1022 > e0 || (int)((m1 >> 52) & 0x7ff) - 1022 > e1;
-            gemm64::digit_bits(gemm64::to_fixed(v[x0], e0), d0);
-            gemm64::digit_bits(gemm64::to_fixed(v[x0 + 1], e1), d1);
+            gemm64::field_digit_bits(gemm64::to_fixed(v[x0], e0), d0);
+            gemm64::field_digit_bits(gemm64::to_fixed(v[x0 + 1], e1), d1);
 #pragma unroll
             for (int p = 0; p < NS; p++) w4[p][u] = d0[p] | (d1[p] << 16);
           }

@@ -19,6 +19,7 @@
 // operand is double-buffered.  Every wait is bounded (DEV_TIMEOUT).
 #include <cuda_bf16.h>
 
+#include "convert.cuh"
 #include "gemm_tc.h"
 #include "tc.cuh"
 #include "trsm_tc.h"
@@ -64,16 +65,12 @@ __device__ inline void raise_timeout(Shared *sh, int *status) {
 
 // x = p0 + p1 + p2 (each BF16, round to nearest): the operand split of the
 // FP32 class.
-template <typename T>
-__device__ inline void split3(T x, uint16_t &p0, uint16_t &p1, uint16_t &p2) {
-  const __nv_bfloat16 b0 = __float2bfloat16_rn((float)x);
-  const T r1 = x - (T)__bfloat162float(b0);
-  const __nv_bfloat16 b1 = __float2bfloat16_rn((float)r1);
-  const T r2 = r1 - (T)__bfloat162float(b1);
-  const __nv_bfloat16 b2 = __float2bfloat16_rn((float)r2);
+__device__ inline void split3(double x, uint16_t &p0, uint16_t &p1, uint16_t &p2) {
+  const __nv_bfloat16 b0 = __float2bfloat16_rn(f32_of(x));
   p0 = __bfloat16_as_ushort(b0);
-  p1 = __bfloat16_as_ushort(b1);
-  p2 = __bfloat16_as_ushort(b2);
+  const double r1 = x - f64_of_bf16(p0);
+  p1 = __bfloat16_as_ushort(__float2bfloat16_rn(f32_of(r1)));
+  p2 = __bfloat16_as_ushort(__float2bfloat16_rn(f32_of(r1 - f64_of_bf16(p1))));
 }
 
 // The three pieces of x0 and x1, packed two per word (x0 in the low half):
@@ -141,7 +138,7 @@ __global__ void k_lkk_prep(const double *__restrict__ t64, const long *__restric
   for (int c = ty; c < 32; c += 8) {
     const size_t o = (size_t)(rb * 32 + tx) + (size_t)(cb * 32 + c) * nb;
     const double x = L[o];
-    L32z[o] = (float)-x;
+    L32z[o] = f32_of(-x);
     blk[tx][c] = x;
   }
   __syncthreads();
