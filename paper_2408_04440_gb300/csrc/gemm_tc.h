@@ -22,7 +22,7 @@ namespace gemm_tc {
 
 constexpr int BM = 128;   // rows of an output block (TMEM lanes)
 constexpr int BN = 256;   // columns of an output block (TMEM columns)
-constexpr int BK = 32;    // K per pipeline stage (BF16: 64 bytes, 64B swizzle)
+constexpr int BK = 32;    // K per slice (BF16: 64 bytes, 64B swizzle); a stage holds one to four
 constexpr int STAGES = 3;
 constexpr int NPIECE = 3; // split pieces of an FP32-class operand
 
@@ -54,9 +54,9 @@ struct Outputs {
 };
 
 // Operand sources of a launch: BF16 pieces (A box 128 x 32, B box 256 x 32,
-// 64-byte swizzle), FP8-E4M3 copies (same boxes in bytes, 32-byte swizzle)
-// with one power-of-two scale per tile, and TF32 copies (FP32 containers,
-// same boxes, 128-byte swizzle).
+// 64-byte swizzle), FP8-E4M3 copies (A box 128 x 128, B box 256 x 128,
+// 128-byte swizzle) with one power-of-two scale per tile, and TF32 copies
+// (FP32 containers, boxes of 32 columns, 128-byte swizzle).
 struct Operands {
   CUtensorMap a16, b16, a8, b8, a32, b32;
   const float *scale8;
@@ -73,7 +73,7 @@ emu_status make_map_bf16_sw128(emu_ctx *ctx, CUtensorMap *map, const void *base,
                                uint32_t box_rows);
 
 // 2-D FP8 tensor map over a row-major [rows x inner] byte array, box
-// [box_rows x 32], 32-byte swizzle.
+// [box_rows x 128], 128-byte swizzle.
 emu_status make_map_e4m3(emu_ctx *ctx, CUtensorMap *map, const void *base, uint64_t inner,
                          uint64_t rows, uint32_t box_rows);
 
