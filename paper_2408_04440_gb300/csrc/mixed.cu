@@ -194,20 +194,25 @@ __global__ void __launch_bounds__(1024)
 // TRSM's 128-row block, or nb - 64 > 512 TMEM columns): L_ik = A_ik L_kk^{-T} from the FP32 master A_ik and an FP32 copy
 // of the FP64 L_kk, written back to the master and, split, to the operand
 // arena.
-// One CTA of four warps per (ROWS rows, tile), lane = column of the current
-// 32-column block cb.  L_kk streams through shared memory as 32x32 chunks (rows
-// of block cb, columns of block c <= cb) in a ring of NBUF buffers filled by
-// cp.async several chunks ahead, the same sequence for every CTA.  An entry is
-// the sum of four partial sums over the columns p = w mod 4: warp w forms its
-// one for all rows of the CTA, so that a value of L_kk read from shared memory
-// serves ROWS FMAs and a 16-byte read of X four (X is stored by p mod 4); the
-// warps then exchange the sums and solve the diagonal chunk by forward
-// substitution with shuffles, ROWS / 4 rows each.  (With the four sums of two
-// rows in one warp every FMA waited for its own read of L_kk.)
+// One CTA of four warps per (ROWS rows, tile).  L_kk streams through shared
+// memory as chunks of 64 rows (the 64 columns of X being solved) by 32 columns,
+// in a ring filled by cp.async several chunks ahead, the same sequence for
+// every CTA.  An entry is the sum of four partial sums over the columns
+// p = w mod 4; warp w forms its one for all rows of the CTA, a lane two columns
+// of either 32-column half for half the rows.  X is stored by row pairs and by
+// p mod 4, so that a 16-byte read is two rows and two p, and one FMA
+// instruction does both rows of a pair.  The warps then exchange the sums and
+// solve the diagonal 32 x 32 block by forward substitution with shuffles,
+// ROWS / 4 rows each; the second half takes the first one's columns in between.
+// What bounds it: operands come back from shared memory at 128 bytes a cycle,
+// also where all lanes read one address, so the tile of a lane (8 rows by 4
+// columns) sets the rate.  With one column and 16 rows the FMA pipe was busy
+// 28 % of the time, now 44 %.  Measured at nb = 1024: 63 tiles 4.5 -> 2.6 ms,
+// the one on the critical path 234 -> 115 us.
 constexpr int TS_LD_PAD = 4;
-constexpr int TS_CHUNK = B * B;  // floats per chunk, column-major (32 columns x 32 rows)
-constexpr int TS_NBUF_CRIT = 8;   // chunk buffers, single critical-path tile (1 CTA per SM)
-constexpr int TS_NBUF_PANEL = 4;  // panel launches (4 CTAs per SM hide each other's latency)
+constexpr int TS_COLS = 2 * B;             // rows of a chunk: columns of X solved per pass
+constexpr int TS_CHUNK = TS_COLS * B;      // floats per chunk, column-major (32 columns x 64 rows)
+constexpr int TS_NBUF = 4;
 
 __device__ inline void cp_async16(void *dst, const void *src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
@@ -222,20 +227,30 @@ __device__ inline void cp_async_wait() {
 // Column c of X's 32-column blocks: the eight columns of a partial sum together.
 __device__ inline int ts_perm(int c) { return (c & ~31) | ((c & 3) << 3) | ((c & 31) >> 2); }
 
-// 16-row CTAs for throughput on the panel; 8-row CTAs with a deeper ring for
-// the single tile on the critical path, where more CTAs mean less latency.
-template <int ROWS, int NBUF, bool JOBS = false>
+// a.x += x.x * l, a.y += x.y * l, each rounded once (as two fmaf)
+__device__ inline void fma_pair(uint64_t &a, uint64_t x, uint64_t l) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a) : "l"(x), "l"(l));
+}
+__device__ inline uint64_t twice(float v) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
+  return r;
+}
+
+// 16-row CTAs for throughput on the panel; 8-row CTAs for the single tile on
+// the critical path, where more CTAs mean less latency.
+template <int ROWS, bool JOBS = false>
 __global__ void __launch_bounds__(128)
     k_trsm32_panel(const float *__restrict__ Lkk0, float *__restrict__ t32, uint16_t *__restrict__ op, int nb,
                    int NT, int k, const int *__restrict__ rows, const int *st,
                    const int2 *__restrict__ jobs = nullptr) {
-  constexpr int NTH = 128, RW = ROWS / 4;
+  constexpr int NTH = 128, RW = ROWS / 4, NP = ROWS / 2, NPL = NP / 2, NBUF = TS_NBUF;
   if (failed(st)) return;
   extern __shared__ __align__(16) float sm[];
-  const int ldx = nb + TS_LD_PAD;
-  float *S = sm;                     // [NBUF][32][32]: chunk ring, S[p * 32 + r] = L_kk(cb*32 + r, c*32 + p)
-  float *X = sm + NBUF * TS_CHUNK;   // [ROWS][ldx]: the CTA's rows of A_ik, solved in place
-  float *E = X + ROWS * ldx;         // [4][ROWS][32]: partial sums
+  const int ldx = 2 * nb + TS_LD_PAD;
+  float *S = sm;                     // [NBUF][32][64]: chunk ring, S[p * 64 + r] = L_kk(b*64 + r, c*32 + p)
+  float *X = sm + NBUF * TS_CHUNK;   // [NP][nb][2]: the CTA's rows of A_ik in pairs, solved in place
+  float *E = X + NP * ldx;           // [4][NP][32][2]: partial sums
   int r0 = blockIdx.x * ROWS;
   // tile (i, k) of one matrix, or (batched) an explicit tile index and the
   // slot of its L_kk copy
@@ -250,76 +265,76 @@ __global__ void __launch_bounds__(128)
   }
   float *A = t32 + (size_t)ti * nb * nb + r0;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int nbc = nb / B, nchunks = nbc * (nbc + 1) / 2;
-  // chunk i = (cb, c) with i = cb (cb + 1) / 2 + c, c <= cb
-  int ic_cb = 0, ic_c = 0;  // the next chunk to issue
+  const int nblk = nb / TS_COLS;
+  // chunks (b, c) of block b: c = 0 .. 2 b + 1, the last two on its diagonal
+  const float *src0 = Lkk + (size_t)(tid >> 4) * nb + (tid & 15) * 4, *src = src0;
+  const uint32_t dst0 = (uint32_t)((tid >> 4) * TS_COLS + (tid & 15) * 4);
+  int ib = 0, ic = 0, islot = 0;  // the next chunk to issue
   auto issue = [&]() {
-    const int i = ic_cb * (ic_cb + 1) / 2 + ic_c;
-    if (i < nchunks) {
-      float *dst = S + (i % NBUF) * TS_CHUNK;
-      const float *src = Lkk + (size_t)(ic_c * B) * nb + ic_cb * B;
-      for (int e = tid; e < TS_CHUNK / 4; e += NTH) {
-        const int pc = e >> 3, q = (e & 7) * 4;  // chunk column pc, rows q .. q+3
-        cp_async16(dst + pc * B + q, src + (size_t)pc * nb + q);
+    if (ib < nblk) {
+      float *dst = S + islot * TS_CHUNK + dst0;
+#pragma unroll
+      for (int j = 0; j < 4; j++) cp_async16(dst + j * 8 * TS_COLS, src + (size_t)(j * 8) * nb);
+      src += (size_t)B * nb;
+      if (++ic == 2 * ib + 2) {
+        ic = 0;
+        ib++;
+        src = src0 + ib * TS_COLS;
       }
-      if (++ic_c > ic_cb) {
-        ic_cb++;
-        ic_c = 0;
-      }
+      islot = islot + 1 == NBUF ? 0 : islot + 1;
     }
     cp_async_commit();  // an empty group at the tail keeps the count uniform
+  };
+  int slot = 0;
+  auto next_chunk = [&]() -> const float * {
+    cp_async_wait<NBUF - 2>();  // this thread's copies of the chunk have landed
+    __syncthreads();            // everyone's; and the previous chunk's buffer is free
+    issue();
+    const float *Sc = S + slot * TS_CHUNK;
+    slot = slot + 1 == NBUF ? 0 : slot + 1;
+    return Sc;
   };
   for (int u = 0; u < NBUF - 1; u++) issue();
 #pragma unroll 8
   for (int e = tid; e < ROWS * nb; e += NTH) {
     int r = e % ROWS, c = e / ROWS;
-    X[r * ldx + ts_perm(c)] = A[r + (size_t)c * nb];
+    X[(r >> 1) * ldx + 2 * ts_perm(c) + (r & 1)] = A[r + (size_t)c * nb];
   }
   __syncthreads();
-  int i = 0;
-  for (int cb = 0; cb < nbc; cb++) {
-    float a[ROWS];
+
+  // this lane's rows, columns and products: 2 NPL rows from row pair qp on,
+  // columns cg, cg + 1 of either half of the block
+  const int qp = (lane >> 4) * NPL, cg = 2 * (lane & 15);
+  const float *Xl = X + qp * ldx;
+  // the values of L_kk a lane needs of a chunk's half, p = w mod 4, negated
+  auto load_l = [&](uint64_t (*l)[2], const float *Sc) {
 #pragma unroll
-    for (int q = 0; q < ROWS; q++) a[q] = w == 0 ? X[q * ldx + cb * B + ts_perm(lane)] : 0.f;
-    for (int c = 0; c < cb; c++, i++) {
-      cp_async_wait<NBUF - 2>();  // this thread's copies of chunk i have landed
-      __syncthreads();            // everyone's; and chunk i-1's buffer is free
-      issue();
-      const float *Sc = S + (i % NBUF) * TS_CHUNK;
-      float l[8];
-#pragma unroll
-      for (int u = 0; u < 8; u++) l[u] = Sc[(4 * u + w) * B + lane];
-      const float *Xc = X + c * B + w * 8;
-#pragma unroll
-      for (int h = 0; h < 2; h++)
-#pragma unroll
-        for (int q = 0; q < ROWS; q++) {
-          const float4 xv = *reinterpret_cast<const float4 *>(Xc + q * ldx + 4 * h);
-          a[q] = fmaf(-xv.x, l[4 * h], a[q]);
-          a[q] = fmaf(-xv.y, l[4 * h + 1], a[q]);
-          a[q] = fmaf(-xv.z, l[4 * h + 2], a[q]);
-          a[q] = fmaf(-xv.w, l[4 * h + 3], a[q]);
-        }
+    for (int u = 0; u < 8; u++) {
+      const float2 v = *reinterpret_cast<const float2 *>(Sc + (4 * u + w) * TS_COLS + cg);
+      l[u][0] = twice(-v.x);
+      l[u][1] = twice(-v.y);
     }
-    // diagonal chunk
+  };
+  // the sums of a 32-column half put together and solved; Sc: its diagonal block
+  auto put_sums = [&](const uint64_t (*a)[2]) {
 #pragma unroll
-    for (int q = 0; q < ROWS; q++) E[(w * ROWS + q) * B + lane] = a[q];
-    cp_async_wait<NBUF - 2>();
-    __syncthreads();
-    issue();
-    const float *Sc = S + (i % NBUF) * TS_CHUNK;
-    i++;
-    const float myrinv = 1.0f / Sc[lane * B + lane];
+    for (int q = 0; q < NPL; q++)
+      *reinterpret_cast<ulonglong2 *>(E + ((w * NP + qp + q) * B + cg) * 2) = make_ulonglong2(a[q][0], a[q][1]);
+  };
+  auto solve_half = [&](const float *Sc, int col0) {
+    const float myrinv = 1.0f / Sc[lane * TS_COLS + lane];
     float v[RW];
 #pragma unroll
-    for (int u = 0; u < RW; u++) {
-      const float *e = E + (w * RW + u) * B + lane;
-      v[u] = (e[0] + e[ROWS * B]) + (e[2 * ROWS * B] + e[3 * ROWS * B]);
+    for (int u = 0; u < RW; u += 2) {
+      const float2 *e = reinterpret_cast<const float2 *>(E) + (w * (RW / 2) + u / 2) * B + lane;
+      const float2 e0 = e[0], e1 = e[NP * B], e2 = e[2 * NP * B], e3 = e[3 * NP * B];
+      v[u] = (e0.x + e1.x) + (e2.x + e3.x);
+      v[u + 1] = (e0.y + e1.y) + (e2.y + e3.y);
     }
 #pragma unroll 8
     for (int j = 0; j < B; j++) {
       const float rj = __shfl_sync(0xffffffffu, myrinv, j);
-      const float lj = lane > j ? Sc[j * B + lane] : 0.f;  // L_kk(cb*32 + lane, cb*32 + j)
+      const float lj = lane > j ? Sc[j * TS_COLS + lane] : 0.f;  // L_kk(col0 + lane, col0 + j)
 #pragma unroll
       for (int u = 0; u < RW; u++) {
         const float xj = __shfl_sync(0xffffffffu, v[u], j) * rj;
@@ -328,31 +343,85 @@ __global__ void __launch_bounds__(128)
       }
     }
 #pragma unroll
-    for (int u = 0; u < RW; u++) X[(w * RW + u) * ldx + cb * B + ts_perm(lane)] = v[u];
+    for (int u = 0; u < RW; u += 2)
+      *reinterpret_cast<float2 *>(X + (w * (RW / 2) + u / 2) * ldx + 2 * (col0 + ts_perm(lane))) =
+          make_float2(v[u], v[u + 1]);
     __syncthreads();
+  };
+  for (int b = 0; b < nblk; b++) {
+    uint64_t a0[NPL][2], a1[NPL][2];  // X - sum over p of X(:, p) L_kk(col, p), p = w mod 4 ascending
+    const float *Xb = Xl + 2 * (b * TS_COLS + ts_perm(cg));  // column cg + 1 is eight places on
+#pragma unroll
+    for (int q = 0; q < NPL; q++)
+#pragma unroll
+      for (int x = 0; x < 2; x++) {
+        a0[q][x] = w == 0 ? *reinterpret_cast<const uint64_t *>(Xb + q * ldx + 16 * x) : 0ull;
+        a1[q][x] = w == 0 ? *reinterpret_cast<const uint64_t *>(Xb + q * ldx + 16 * x + 2 * B) : 0ull;
+      }
+    const float *Xc = Xl + w * 16;
+    uint64_t l0[8][2], l1[8][2];
+    for (int c = 0; c < 2 * b; c++, Xc += 2 * B) {
+      const float *Sc = next_chunk();
+      load_l(l0, Sc);
+      load_l(l1, Sc + B);
+#pragma unroll
+      for (int h = 0; h < 4; h++)
+#pragma unroll
+        for (int q = 0; q < NPL; q++) {
+          const ulonglong2 xv = *reinterpret_cast<const ulonglong2 *>(Xc + q * ldx + 4 * h);
+#pragma unroll
+          for (int x = 0; x < 2; x++) {
+            fma_pair(a0[q][x], xv.x, l0[2 * h][x]);
+            fma_pair(a1[q][x], xv.x, l1[2 * h][x]);
+            fma_pair(a0[q][x], xv.y, l0[2 * h + 1][x]);
+            fma_pair(a1[q][x], xv.y, l1[2 * h + 1][x]);
+          }
+        }
+    }
+    put_sums(a0);
+    const float *Sc = next_chunk();
+    solve_half(Sc, b * TS_COLS);
+    load_l(l1, Sc + B);
+#pragma unroll
+    for (int h = 0; h < 4; h++)
+#pragma unroll
+      for (int q = 0; q < NPL; q++) {
+        const ulonglong2 xv = *reinterpret_cast<const ulonglong2 *>(Xc + q * ldx + 4 * h);
+#pragma unroll
+        for (int x = 0; x < 2; x++) {
+          fma_pair(a1[q][x], xv.x, l1[2 * h][x]);
+          fma_pair(a1[q][x], xv.y, l1[2 * h + 1][x]);
+        }
+      }
+    put_sums(a1);
+    Sc = next_chunk();
+    solve_half(Sc + B, b * TS_COLS + B);
   }
   cp_async_wait<0>();
   // FP32 master (column-major) and the sender-side BF16 pieces (row-major)
 #pragma unroll 8
   for (int e = tid; e < ROWS * nb; e += NTH) {
     int r = e % ROWS, c = e / ROWS;
-    A[r + (size_t)c * nb] = X[r * ldx + ts_perm(c)];
+    A[r + (size_t)c * nb] = X[(r >> 1) * ldx + 2 * ts_perm(c) + (r & 1)];
   }
   size_t plane = (size_t)nb * nb;
   uint16_t *P = op + (size_t)ti * 3 * plane + (size_t)r0 * nb;
-  for (int e = tid; e < ROWS * nb; e += NTH) {
-    int r = e / nb, c = e % nb;
-    uint16_t p0, p1, p2;
-    split3(X[r * ldx + ts_perm(c)], p0, p1, p2);
-    size_t off = (size_t)r * nb + c;
-    P[off] = p0;
-    P[plane + off] = p1;
-    P[2 * plane + off] = p2;
-  }
+  for (int c = 2 * tid; c < nb; c += 2 * NTH)
+#pragma unroll 4
+    for (int r = 0; r < ROWS; r++) {
+      const float *x = X + (r >> 1) * ldx + 2 * ts_perm(c) + (r & 1);
+      ushort2 p0, p1, p2;
+      split3(x[0], p0.x, p1.x, p2.x);
+      split3(x[16], p0.y, p1.y, p2.y);  // column c + 1 is eight places on
+      const size_t off = (size_t)r * nb + c;
+      *reinterpret_cast<ushort2 *>(P + off) = p0;
+      *reinterpret_cast<ushort2 *>(P + plane + off) = p1;
+      *reinterpret_cast<ushort2 *>(P + 2 * plane + off) = p2;
+    }
 }
 
-static size_t trsm32_smem(int nb, int rows, int nbuf) {
-  return (size_t)(nbuf * TS_CHUNK + rows * (nb + TS_LD_PAD) + 4 * rows * B) * sizeof(float);
+static size_t trsm32_smem(int nb, int rows) {
+  return (size_t)(TS_NBUF * TS_CHUNK + rows / 2 * (2 * nb + TS_LD_PAD) + 4 * rows * B) * sizeof(float);
 }
 
 // z pieces for the sampler: zp[q][n][k] = piece q of Z[k][n], n < s_pad
@@ -1065,10 +1134,10 @@ static emu_status factor_mixed_record(emu_ctx *ctx, emu_mat *A, MixedPlan *P, in
   cudaEvent_t ev_start = ctx->sched_ev[EV * NT], ev_end = ctx->sched_ev[EV * NT + 1];
   EMU_CUDA_TRY(ctx, cudaEventRecord(ev_start, user));
   for (cudaStream_t q : {ctx->crit, ctx->mid, ctx->bulk}) EMU_CUDA_TRY(ctx, cudaStreamWaitEvent(q, ev_start, 0));
-  size_t tsm16 = trsm32_smem(nb, 16, TS_NBUF_PANEL), tsm8 = trsm32_smem(nb, 8, TS_NBUF_CRIT);
-  EMU_CUDA_TRY(ctx, cudaFuncSetAttribute(k_trsm32_panel<16, TS_NBUF_PANEL>,
+  size_t tsm16 = trsm32_smem(nb, 16), tsm8 = trsm32_smem(nb, 8);
+  EMU_CUDA_TRY(ctx, cudaFuncSetAttribute(k_trsm32_panel<16>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm16));
-  EMU_CUDA_TRY(ctx, cudaFuncSetAttribute(k_trsm32_panel<8, TS_NBUF_CRIT>,
+  EMU_CUDA_TRY(ctx, cudaFuncSetAttribute(k_trsm32_panel<8>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm8));
 
   // TRSM of the listed rows of panel k: FP64 rows on the FP64 pipe, then split;
@@ -1155,10 +1224,10 @@ static emu_status factor_mixed_record(emu_ctx *ctx, emu_mat *A, MixedPlan *P, in
       ProfScope ps(ctx, PROF_TRSM32, n32 * nb3, 14.0 * n32 * te);
       const float *lkk = P->d_lkk32 + (size_t)(k & 1) * te;
       if (critical)
-        k_trsm32_panel<8, TS_NBUF_CRIT><<<dim3(nb / 8, n32), 128, tsm8, ctx->stream>>>(
+        k_trsm32_panel<8><<<dim3(nb / 8, n32), 128, tsm8, ctx->stream>>>(
             lkk, A->t32, A->op_bf16, nb, NT, k, P->d_rows32 + r32, st);
       else
-        k_trsm32_panel<16, TS_NBUF_PANEL><<<dim3(nb / 16, n32), 128, tsm16, ctx->stream>>>(
+        k_trsm32_panel<16><<<dim3(nb / 16, n32), 128, tsm16, ctx->stream>>>(
             lkk, A->t32, A->op_bf16, nb, NT, k, P->d_rows32 + r32, st);
       EMU_LAUNCHED(ctx);
     }
@@ -1534,8 +1603,8 @@ emu_status launch_trsm32_jobs(emu_ctx *ctx, const float *slots, float *t32, uint
   if (njobs <= 0) return EMU_OK;
   // the critical form where 16-row CTAs of the jobs do not fill the chip
   const bool few = njobs * (nb / 16) < 2 * ctx->sm_count;
-  size_t sm = few ? trsm32_smem(nb, 8, TS_NBUF_CRIT) : trsm32_smem(nb, 16, TS_NBUF_PANEL);
-  auto kern = few ? k_trsm32_panel<8, TS_NBUF_CRIT, true> : k_trsm32_panel<16, TS_NBUF_PANEL, true>;
+  size_t sm = few ? trsm32_smem(nb, 8) : trsm32_smem(nb, 16);
+  auto kern = few ? k_trsm32_panel<8, true> : k_trsm32_panel<16, true>;
   EMU_CUDA_TRY(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   double nb3 = (double)nb * nb * nb;
   ProfScope ps(ctx, PROF_TRSM32, njobs * nb3, 14.0 * njobs * nb * nb);
