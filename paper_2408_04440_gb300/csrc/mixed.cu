@@ -425,21 +425,35 @@ static size_t trsm32_smem(int nb, int rows) {
 }
 
 // z pieces for the sampler: zp[q][n][k] = piece q of Z[k][n], n < s_pad
-// (zero beyond s).
-__global__ void k_split_z(const double *__restrict__ Z, long ldz, long npad, int s, int s_pad,
-                          uint16_t *__restrict__ zp) {
-  long total = npad * (long)s_pad;
-  size_t plane = (size_t)s_pad * npad;
-  for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < total; q += (long)gridDim.x * blockDim.x) {
-    long k = q % npad;
-    int n = (int)(q / npad);
-    double x = (n < s) ? Z[k + (size_t)n * ldz] : 0.0;
-    uint16_t p0, p1, p2;
-    split3(x, p0, p1, p2);
-    zp[q] = p0;
-    zp[plane + q] = p1;
-    zp[2 * plane + q] = p2;
+// (zero beyond s).  A thread takes four rows of column blockIdx.y, so that a
+// piece of them is one 8-byte store (npad is a multiple of 64; Z may start
+// and step by any number of doubles); a 64-bit division per element to find
+// its column took longer than the memory traffic.  16384 x 1024: 219 -> 68 us.
+__global__ void __launch_bounds__(256)
+    k_split_z(const double *__restrict__ Z, long ldz, long npad, int s, int s_pad, uint16_t *__restrict__ zp) {
+  const size_t plane = (size_t)s_pad * npad;
+  const long k = 4 * (blockIdx.x * (long)blockDim.x + threadIdx.x);
+  if (k >= npad) return;
+  for (int n = blockIdx.y; n < s_pad; n += gridDim.y) {
+    ushort4 p0{}, p1{}, p2{};
+    if (n < s) {
+      const double *z = Z + k + (size_t)n * ldz;
+      const double x0 = z[0], x1 = z[1], x2 = z[2], x3 = z[3];
+      split3(x0, p0.x, p1.x, p2.x);
+      split3(x1, p0.y, p1.y, p2.y);
+      split3(x2, p0.z, p1.z, p2.z);
+      split3(x3, p0.w, p1.w, p2.w);
+    }
+    uint16_t *d = zp + (size_t)n * npad + k;
+    *reinterpret_cast<ushort4 *>(d) = p0;
+    *reinterpret_cast<ushort4 *>(d + plane) = p1;
+    *reinterpret_cast<ushort4 *>(d + 2 * plane) = p2;
   }
+}
+
+// Grid of k_split_z.
+static dim3 split_z_grid(long npad, int s_pad) {
+  return dim3((unsigned)((npad + 1023) / 1024), (unsigned)std::min(s_pad, 65535));
 }
 
 }  // namespace
@@ -1345,7 +1359,7 @@ void mixed_fill_info(const emu_mat *A, emu_factor_info *info) {
   }
 }
 
-// Y = L Z: FP64-class tiles on the FP64 pipe (this also initialises Y), the
+// Y = L Z: FP64-class tiles as digit products (this also initialises Y), the
 // FP32/BF16-class tiles on the tensor cores accumulated in FP32 per output
 // block over k in a fixed order, then added to Y.
 // Digit slices of the factor's FP64-class tiles for the sampler, with one
@@ -1503,7 +1517,7 @@ emu_status mixed_sample(emu_ctx *ctx, const emu_mat *L, const double *Z, long ld
   EMU_CUDA_TRY(ctx, cudaMemcpyAsync(d_segs, segs.data(), sbytes, cudaMemcpyHostToDevice, ctx->stream));
   {
     ProfScope ps(ctx, PROF_SPLIT, 0.0, 14.0 * npad * s_pad);
-    k_split_z<<<8 * ctx->sm_count, 256, 0, ctx->stream>>>(Z, ldz, npad, s, s_pad, zp);
+    k_split_z<<<split_z_grid(npad, s_pad), 256, 0, ctx->stream>>>(Z, ldz, npad, s, s_pad, zp);
     EMU_LAUNCHED(ctx);
   }
   double tf = 0.0, tm = 0.0;
@@ -1635,7 +1649,7 @@ emu_status launch_quant_e4m3(emu_ctx *ctx, const uint16_t *op, uint8_t *op8, flo
 
 emu_status launch_split_z(emu_ctx *ctx, const double *Z, long ldz, long npad, int s, int s_pad, uint16_t *zp) {
   ProfScope ps(ctx, PROF_SPLIT, 0.0, 14.0 * npad * s_pad);
-  k_split_z<<<8 * ctx->sm_count, 256, 0, ctx->stream>>>(Z, ldz, npad, s, s_pad, zp);
+  k_split_z<<<split_z_grid(npad, s_pad), 256, 0, ctx->stream>>>(Z, ldz, npad, s, s_pad, zp);
   EMU_LAUNCHED(ctx);
   return EMU_OK;
 }
