@@ -25,28 +25,48 @@ namespace {
 __device__ inline bool failed(const int *st) { return *((volatile const int *)st) != DEV_OK; }
 
 // f_t = sum_p phi_p f_{t-p} + xi_t per coefficient (f before t = 0 is zero):
-// one thread per coefficient, the P previous values in registers.
-constexpr int kMaxP = 8;
-__global__ void k_var(const double *__restrict__ xi, long ldxi, int n, int T, const double *__restrict__ phi, int P,
-                      double *__restrict__ f, long ldf, const int *st) {
+// one thread per coefficient, the KP previous values in registers.  The
+// recursion is a serial chain of FP64 operations, which an SM issues one warp
+// of every 19 cycles or so: KP is P itself up to four lags instead of kMaxP
+// throughout, CTAs of one warp spread the coefficients over all SMs, and the
+// inputs are read eight steps ahead.  16384 coefficients, 256 steps, P = 3:
+// 162 -> 120 us.
+constexpr int kMaxP = 8, kVarAhead = 8;
+template <int KP>
+__global__ void __launch_bounds__(32)
+    k_var(const double *__restrict__ xi, long ldxi, int n, int T, const double *__restrict__ phi, int P,
+          double *__restrict__ f, long ldf, const int *st) {
   if (failed(st)) return;
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
-  double c[kMaxP], h[kMaxP];
+  double c[KP], h[KP], x[kVarAhead];
 #pragma unroll
-  for (int p = 0; p < kMaxP; p++) {
+  for (int p = 0; p < KP; p++) {
     c[p] = p < P ? phi[k + (long)p * n] : 0.0;
     h[p] = 0.0;  // h[p] = f_{t-1-p}
   }
-  for (int t = 0; t < T; t++) {
-    double v = 0.0;
 #pragma unroll
-    for (int p = 0; p < kMaxP; p++) v = fma(c[p], h[p], v);
-    v += xi[k + (long)t * ldxi];
+  for (int u = 0; u < kVarAhead; u++) x[u] = u < T ? xi[k + (long)u * ldxi] : 0.0;
+  unsigned bad = 0;  // bit p: f_{t-1-p} is not finite
+  for (int t0 = 0; t0 < T; t0 += kVarAhead) {
 #pragma unroll
-    for (int p = kMaxP - 1; p > 0; p--) h[p] = h[p - 1];
-    h[0] = v;
-    f[k + (long)t * ldf] = v;
+    for (int u = 0; u < kVarAhead; u++) {
+      const int t = t0 + u;
+      if (t >= T) break;
+      const double xt = x[u];
+      if (t + kVarAhead < T) x[u] = xi[k + (long)(t + kVarAhead) * ldxi];
+      double v = xt;  // the newest value last: one FMA of latency per step
+#pragma unroll
+      for (int p = KP - 1; p >= 0; p--) v = fma(c[p], h[p], v);
+      // kMaxP lags count: a value that is not finite is NaN against the zero
+      // factors of lags KP + 1 .. kMaxP too
+      if (bad & ((1u << kMaxP) - (1u << KP))) v = __longlong_as_double(0x7ff8000000000000ll);
+      bad = bad << 1 | ((__double2hiint(v) & 0x7ff00000) == 0x7ff00000);
+#pragma unroll
+      for (int p = KP - 1; p > 0; p--) h[p] = h[p - 1];
+      h[0] = v;
+      f[k + (long)t * ldf] = v;
+    }
   }
 }
 
@@ -456,7 +476,8 @@ emu_status emu_var_recursion(emu_ctx *ctx, const double *dXi, int n, int T, long
     return EMU_EINVAL;
   EMU_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
   EMU_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, ST_WORDS * sizeof(int), ctx->stream));
-  k_var<<<(n + 127) / 128, 128, 0, ctx->stream>>>(dXi, ldxi, n, T, dPhi, P, dF, ldf, ctx->d_status);
+  auto var = P == 1 ? k_var<1> : P == 2 ? k_var<2> : P == 3 ? k_var<3> : P == 4 ? k_var<4> : k_var<kMaxP>;
+  var<<<(n + 31) / 32, 32, 0, ctx->stream>>>(dXi, ldxi, n, T, dPhi, P, dF, ldf, ctx->d_status);
   EMU_LAUNCHED(ctx);
   EMU_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
   return EMU_OK;
