@@ -1769,8 +1769,13 @@ emu_status launch_potrf64_ptr(emu_ctx *ctx, double *D, int nb, int k) {
   double *rinv = reinterpret_cast<double *>(ctx->dag_ws + dag_ws_ints(nbb, 1));
   if (ctx->dag_clus == 1) {
     // the chain on cluster 0 (three CTAs), the tasks on the other clusters;
-    // two workers per SM: the task throughput paces the chain
-    int g = ctx->dag_ntasks + 2 < 2 * ctx->sm_count ? ctx->dag_ntasks + 2 : 2 * ctx->sm_count;
+    // the task throughput paces the chain: two workers per SM, three above
+    // nb = 512, where the tasks (nb^3) outgrow the chain (nb).  One tile with
+    // 2 / 3 workers: nb = 512 259 / 261 us (a factor at n = 16384 15.8 / 16.2
+    // ms), nb = 768 475 / 421, nb = 1024 912 / 742 (four: 695, but the n =
+    // 22500 class-format factor takes 48.7 ms instead of 48.1)
+    const int workers = (nbb > 32 ? 3 : 2) * ctx->sm_count;
+    int g = ctx->dag_ntasks + 2 < workers ? ctx->dag_ntasks + 2 : workers;
     g = (g + 2) / 3 * 3;
     if (g < 6) g = 6;
     cudaLaunchConfig_t cfg = {};
