@@ -322,11 +322,11 @@ TRAFFIC = {("tc_factor", 128, 512, 1e-8, MASK_FP64_FP32_BF16): 99.6e6}
 
 ALU_NOTES = {
     "potrf": "the diagonal-tile POTRF is bound by its FP64 dependency chain (one 16-column leaf after another)",
-    "update64": "FP64 tile updates are FP64-pipe bound; their launch times include sharing the SMs with the "
-                "concurrent streams",
+    "update64": "FP64 tile updates of tile sizes that are not a multiple of 128 are FP64-pipe bound; their launch "
+                "times include sharing the SMs with the concurrent streams",
     "trsm64": "the FP64 panel TRSM is bound by its substitution chain and by the SMs left beside the bulk update",
-    "trmm64": "FP64-class tiles of the sampler, FP64-pipe bound",
-    "solve": "triangular solves, bound by their substitution chains",
+    "trmm64": "draws of a plain FP64 factor whose tile size is not a multiple of 128, FP64-pipe bound",
+    "solve": "triangular solves, bound by the chain of their diagonal blocks",
     "trsm32": "the SIMT FP32 panel TRSM (tile sizes whose trailing columns do not fit in TMEM) is bound by its "
               "substitution chain and by L_kk strip loads, on the SMs left beside the bulk update",
 }
@@ -715,8 +715,8 @@ def cfg3_e4m3_refine(E, ctx) -> dict:
     out["fp64_class_tc_backward_error_est"] = E.emu_backward_error_est(ctx, A, L, beta, nprobes=8, seed=5)
     out["speedup_vs_fp64_class_tc"] = round(i64.ms / ms[-1], 2)
     A.free()
-    out["fp64_pipe"] = ("not run in the default bench (about 80 s at the DFMA rate); see --workload fp64_L400 "
-                        "for the plain FP64 factor at scale")
+    out["fp64_pipe"] = ("not run: the plain FP64 factor of this tile size runs as digit products too; see --workload "
+                        "fp64_L400 for it at scale")
     return out
 
 
@@ -804,7 +804,7 @@ def fp64tc_headline(E, ctx, a, flops, mixed_ms) -> dict:
         A.free()
     return {"factor_ms": round(ms[-1], 3), "tflops": round(flops / (ms[-1] * 1e-3) / 1e12, 3),
             "backward_error_est": est, "speedup_of_mixed": round(ms[-1] / mixed_ms, 2),
-            "note": "FP64-accurate factor on the tensor cores (Ozaki digits); the plain FP64 row is the FP64 pipe"}
+            "note": "FP64-class tiles in the mixed factor's schedule (Ozaki digits); the plain FP64 row is the FP64 factor"}
 
 
 def other_configs(E, ctx, a, flops, mixed_ms) -> dict:
@@ -1100,7 +1100,7 @@ def run_reference_batched(a):
 
 
 def run_fp64_L400(a):
-    """The FP64 comparison at L=400 (n=160000, nb=1024, beta=16): the plain FP64 tile Cholesky on the FP64 pipe
+    """The FP64 comparison at L=400 (n=160000, nb=1024, beta=16): the plain FP64 tile Cholesky
     (about 104 GB of FP64 lower tiles) and the same factor with every tile FP64-class on the tensor cores in
     class-format storage, each once, with the SM clocks sampled meanwhile."""
     import torch

@@ -415,7 +415,10 @@ emu_status emu_mat_free(emu_mat *A);
 
 /* ------------------------------------------------------------------ factor */
 /* Factor A = L L^T in place (A must hold a covariance, state 0).  Plain FP64
- * when o == NULL or o->eps <= 0, otherwise the adaptive mixed-precision tile
+ * when o == NULL or o->eps <= 0 (with nb a multiple of 128 the trailing updates
+ * and block products are formed on the tensor cores with FP64 accuracy, exact
+ * digit products rounded once; where their workspace does not fit, and for
+ * other nb, in FP64 arithmetic), otherwise the adaptive mixed-precision tile
  * factor described at emu_mp_opts.  On a non-positive pivot returns
  * EMU_ENOTPD with info->pivot set and leaves A in an unspecified state. */
 emu_status emu_potrf_mp(emu_ctx *ctx, emu_mat *A, const emu_mp_opts *o,
@@ -448,14 +451,16 @@ emu_status emu_sample_host(emu_ctx *ctx, const emu_mat *L, int nsamples,
  * of their FP64 factor tiles, the off-diagonal tiles as stored (FP64 tiles
  * rounded to FP32, FP32 masters as they are), each tile's product accumulated
  * in FP32 and added to the FP64 right-hand sides (it is the preconditioner of
- * emu_solve_refine, whose residual and update are FP64).  dB, dX: n x nrhs,
+ * emu_solve_refine, whose residual has FP64 accuracy and whose update is FP64).  dB, dX: n x nrhs,
  * column-major; dX may equal dB. */
 emu_status emu_potrs(emu_ctx *ctx, const emu_mat *L, const double *dB,
                      long ldb, double *dX, long ldx, int nrhs);
 
 /* Solve S X = B by iterative refinement: X0 = (L L^T)^{-1} B, then FP64
  * residual R = B - S X against the FP64 covariance S (state 0, same n and
- * nb as L), correction D = (L L^T)^{-1} R in the factor's precisions, FP64
+ * nb as L; in FP64 arithmetic, or with the same accuracy from exact digit
+ * products on the tensor cores for several right-hand sides and up to 20000
+ * padded rows), correction D = (L L^T)^{-1} R in the factor's precisions, FP64
  * update X += D, until every column's normwise backward error
  * ||r||_2 / (||S||_F ||x||_2 + ||b||_2) is <= tol.  Returns EMU_ENOCONV when
  * maxit corrections do not reach tol (X then holds the last iterate). */
