@@ -29,9 +29,10 @@ __device__ inline bool failed(const int *st) { return *((volatile const int *)st
 // recursion is a serial chain of FP64 operations, which an SM issues one warp
 // of every 19 cycles or so: KP is P itself up to four lags instead of kMaxP
 // throughout, CTAs of one warp spread the coefficients over all SMs, and the
-// inputs are read eight steps ahead.  16384 coefficients, 256 steps, P = 3:
-// 162 -> 120 us.
-constexpr int kMaxP = 8, kVarAhead = 8;
+// inputs of the next kVarAhead steps are read together while these run (read
+// one per step, that far ahead, each step waited for the youngest load: 120
+// us).  16384 coefficients, 256 steps, P = 3: 162 -> 36 us.
+constexpr int kMaxP = 8, kVarAhead = 16;
 template <int KP>
 __global__ void __launch_bounds__(32)
     k_var(const double *__restrict__ xi, long ldxi, int n, int T, const double *__restrict__ phi, int P,
@@ -39,23 +40,27 @@ __global__ void __launch_bounds__(32)
   if (failed(st)) return;
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
-  double c[KP], h[KP], x[kVarAhead];
+  double c[KP], h[KP], x[kVarAhead], next[kVarAhead];
 #pragma unroll
   for (int p = 0; p < KP; p++) {
     c[p] = p < P ? phi[k + (long)p * n] : 0.0;
     h[p] = 0.0;  // h[p] = f_{t-1-p}
   }
 #pragma unroll
-  for (int u = 0; u < kVarAhead; u++) x[u] = u < T ? xi[k + (long)u * ldxi] : 0.0;
+  for (int u = 0; u < kVarAhead; u++) next[u] = u < T ? xi[k + (long)u * ldxi] : 0.0;
   unsigned bad = 0;  // bit p: f_{t-1-p} is not finite
   for (int t0 = 0; t0 < T; t0 += kVarAhead) {
 #pragma unroll
     for (int u = 0; u < kVarAhead; u++) {
+      x[u] = next[u];
+      const int t = t0 + kVarAhead + u;
+      next[u] = t < T ? xi[k + (long)t * ldxi] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < kVarAhead; u++) {
       const int t = t0 + u;
       if (t >= T) break;
-      const double xt = x[u];
-      if (t + kVarAhead < T) x[u] = xi[k + (long)(t + kVarAhead) * ldxi];
-      double v = xt;  // the newest value last: one FMA of latency per step
+      double v = x[u];  // the newest value last: one FMA of latency per step
 #pragma unroll
       for (int p = KP - 1; p >= 0; p--) v = fma(c[p], h[p], v);
       // kMaxP lags count: a value that is not finite is NaN against the zero

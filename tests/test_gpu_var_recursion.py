@@ -1,6 +1,6 @@
 """The lagged recursion f_t = sum_p phi_p f_{t-p} + xi_t against NumPy: every
 number of lags (the kernel is compiled per lag count up to four), sizes around
-a warp and the eight steps read ahead, and values that are not finite."""
+a warp and the sixteen steps read ahead, and values that are not finite."""
 import numpy as np
 import pytest
 
@@ -39,7 +39,7 @@ def _run(xi, phi):
 
 
 @pytest.mark.parametrize("P", range(1, 9))
-@pytest.mark.parametrize("n,T", [(1, 1), (31, 7), (33, 8), (1000, 9), (64, 41)])
+@pytest.mark.parametrize("n,T", [(1, 1), (31, 7), (33, 8), (1000, 9), (64, 41), (65, 15), (5, 16), (32, 17), (3, 33)])
 def test_matches_numpy(P, n, T):
     xi, phi = _case(P, n, T, 100 * P + T)
     ref = _recursion(xi, phi)
