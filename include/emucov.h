@@ -451,16 +451,14 @@ emu_status emu_sample_host(emu_ctx *ctx, const emu_mat *L, int nsamples,
  * of their FP64 factor tiles, the off-diagonal tiles as stored (FP64 tiles
  * rounded to FP32, FP32 masters as they are), each tile's product accumulated
  * in FP32 and added to the FP64 right-hand sides (it is the preconditioner of
- * emu_solve_refine, whose residual has FP64 accuracy and whose update is FP64).  dB, dX: n x nrhs,
+ * emu_solve_refine, whose residual and update are FP64).  dB, dX: n x nrhs,
  * column-major; dX may equal dB. */
 emu_status emu_potrs(emu_ctx *ctx, const emu_mat *L, const double *dB,
                      long ldb, double *dX, long ldx, int nrhs);
 
 /* Solve S X = B by iterative refinement: X0 = (L L^T)^{-1} B, then FP64
  * residual R = B - S X against the FP64 covariance S (state 0, same n and
- * nb as L; in FP64 arithmetic, or with the same accuracy from exact digit
- * products on the tensor cores for several right-hand sides and up to 20000
- * padded rows), correction D = (L L^T)^{-1} R in the factor's precisions, FP64
+ * nb as L), correction D = (L L^T)^{-1} R in the factor's precisions, FP64
  * update X += D, until every column's normwise backward error
  * ||r||_2 / (||S||_F ||x||_2 + ||b||_2) is <= tol.  Returns EMU_ENOCONV when
  * maxit corrections do not reach tol (X then holds the last iterate). */

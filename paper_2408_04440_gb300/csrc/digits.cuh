@@ -58,20 +58,6 @@ __device__ inline void digit_bits(long long X, uint32_t (&d)[NS]) {
     d[p] = __float_as_uint(__int_as_float(0x4B400000 + (int)dg) - 12582912.0f) >> 16;
   }
 }
-// Digits with the same bounds and sum (-64 <= digit p < 64 for p >= 1) at a
-// third of the instructions: with 64 added at every digit but the first, the
-// biased digits are the 7-bit fields of X.
-__device__ inline void field_digit_bits(long long X, uint32_t (&d)[NS]) {
-  constexpr long long kBias = 0x1020408102040LL;  // sum of 64 2^(7 q), q = 0 .. NS - 2
-  const long long Y = X + kBias;
-  const int top = (int)(Y >> (SLICE_BITS * (NS - 1)));
-  d[0] = __float_as_uint(__int_as_float(0x4B400000 + top) - 12582912.0f) >> 16;
-#pragma unroll
-  for (int p = 1; p < NS; p++) {
-    const uint32_t f = (uint32_t)((unsigned long long)Y >> (SLICE_BITS * (NS - 1 - p))) & 127u;
-    d[p] = __float_as_uint(__uint_as_float(0x4B000000u | f) - 8388672.0f) >> 16;
-  }
-}
 // Digits of v with row exponent e written d[0], d[plane], ...
 __device__ inline void write_digits(double v, int e, uint16_t *d, size_t plane) {
   uint32_t g[NS];

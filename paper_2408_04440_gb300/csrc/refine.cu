@@ -8,7 +8,7 @@
 #include <vector>
 
 #include "mixed.h"
-#include "symm_digits.h"
+#include "refine_split.h"
 
 namespace {
 
@@ -19,9 +19,13 @@ namespace {
 // through shared memory in 32-wide K chunks so that every global read is
 // coalesced.  part[z][row][P] of range z and group blockIdx.z; deterministic:
 // one CTA owns each partial sum, k_symm_finish adds the ranges in order.
-// P follows the right-hand sides (one of them cost sixteen columns' FP64 work),
-// and the ranges fill the chip where n / 64 slabs do not (60 CTAs at n = 3840).
-constexpr int RS = 64, RK = 32;
+//
+// Bound by FP64 issue from a few right-hand sides on.  As digit products on the
+// tensor cores n = 16384 with 16 columns takes 1.5 ms instead of 7.3, but that
+// cuts the entries of S relative to their tile: a solution's entry that hangs on
+// covariances 1e-12 of their tile's largest was off by 1.5e-6 of itself after
+// refinement, where this sum, which takes every entry of S whole, leaves 5e-15.
+constexpr int RK = 32;
 template <int P>
 __global__ void __launch_bounds__(256)
     k_symm_part(const double *__restrict__ t64, int nb, int NT, const double *__restrict__ X, double *__restrict__ part,
@@ -144,23 +148,11 @@ __global__ void k_axpy(double *__restrict__ X, const double *__restrict__ D, lon
 
 }  // namespace
 
-// Right-hand sides per group, groups and column ranges of the product.
-struct SymmShape {
-  int P, groups, nz;
-};
-static SymmShape symm_shape(const emu_ctx *ctx, const emu_mat *S, int nrhs) {
-  SymmShape s;
-  s.P = nrhs == 1 ? 1 : nrhs <= 4 ? 4 : nrhs <= 8 ? 8 : nrhs <= 16 ? 16 : 32;
-  s.groups = (nrhs + s.P - 1) / s.P;
-  const int slabs = S->nt * (S->nb / RS) * s.groups;
-  s.nz = std::max(1, std::min(S->nt, (6 * ctx->sm_count + slabs - 1) / slabs));
-  return s;
-}
 // R = B - S X (npad x nrhs each); part: groups nz npad P doubles.
 static emu_status symm_residual(emu_ctx *ctx, const emu_mat *S, const double *X, const double *Bp, double *R,
                                 double *part, int nrhs) {
   const long npad = (long)S->nt * S->nb;
-  const SymmShape sh = symm_shape(ctx, S, nrhs);
+  const ResidualSplit sh = residual_split(ctx->sm_count, S->nt, S->nb, nrhs);
   ProfScope ps(ctx, PROF_SOLVE, 2.0 * (double)npad * npad * nrhs, 8.0 * (double)npad * npad);
   const dim3 grid((unsigned)(npad / RS), (unsigned)sh.nz, (unsigned)sh.groups);
   auto kern = sh.P == 1    ? k_symm_part<1>
@@ -175,8 +167,6 @@ static emu_status symm_residual(emu_ctx *ctx, const emu_mat *S, const double *X,
   return EMU_OK;
 }
 
-constexpr long kDigitResidualRows = 20000;
-
 emu_status refine_solve(emu_ctx *ctx, const emu_mat *L, const emu_mat *S, const double *dB,
                         long ldb, double *dX, long ldx, int nrhs, double tol, int maxit,
                         emu_refine_info *info) {
@@ -185,20 +175,9 @@ emu_status refine_solve(emu_ctx *ctx, const emu_mat *L, const emu_mat *S, const 
   long npad = (long)L->nt * L->nb;
   size_t blk = (size_t)npad * nrhs;
   double *buf = nullptr, *norms = nullptr;
-  // The residual's product: as digit products from two right-hand sides and
-  // 2048 rows on (n = 16384, 16 columns: 7.3 -> 1.5 ms; one column is bound by
-  // the tiles' memory traffic either way); on the FP64 pipe otherwise, and when
-  // a bound of the digits does not hold (*flag).  Above kDigitResidualRows the
-  // FP64 pipe stays, although the product takes 116 ms there instead of 23 (n =
-  // 65536): a solution that stops at 1e-12 there carries the rounding of that
-  // residual, and moved by 1.7e-9 with the more exact one (n = 16384: 3e-12).
-  bool digits = symm_digits::supports(S) && nrhs >= 2 && npad >= 2048 && npad <= kDigitResidualRows;
-  const SymmShape sh = symm_shape(ctx, S, nrhs);
-  symm_digits::Plan dp = symm_digits::shape(ctx, S, nrhs);
-  const size_t part = std::max((size_t)sh.groups * sh.nz * npad * sh.P,
-                               digits ? (size_t)dp.groups * dp.nz * npad * symm_digits::NR : 0);
-  const size_t ws = (4 * blk + part) * sizeof(double), ws_pad = (ws + 255) & ~(size_t)255;
-  EMU_CUDA_TRY(ctx, cudaMallocAsync(&buf, ws_pad + (digits ? symm_digits::bytes(S) : 0), ctx->stream));
+  const ResidualSplit sh = residual_split(ctx->sm_count, S->nt, S->nb, nrhs);
+  const size_t part = (size_t)sh.groups * sh.nz * npad * sh.P;
+  EMU_CUDA_TRY(ctx, cudaMallocAsync(&buf, (4 * blk + part) * sizeof(double), ctx->stream));
   EMU_CUDA_TRY(ctx, cudaMallocAsync(&norms, 3 * nrhs * sizeof(double), ctx->stream));
   double *Bp = buf, *X = buf + blk, *R = buf + 2 * blk, *D = buf + 3 * blk;
   std::vector<double> hn(3 * nrhs);
@@ -214,38 +193,22 @@ emu_status refine_solve(emu_ctx *ctx, const emu_mat *L, const emu_mat *S, const 
   if (e == cudaSuccess) e = cudaMemcpyAsync(&frobS, S->d_frob, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
   if (e == cudaSuccess) e = cudaEventRecord(ctx->ev0, ctx->stream);
   if (e != cudaSuccess) s = emu_cuda_fail(ctx, e, "refine setup");
-  int hflag = 0;
-  if (s == EMU_OK && digits) s = symm_digits::init(ctx, &dp, reinterpret_cast<char *>(buf) + ws_pad, S);
   // X0 = M^{-1} B
   if (s == EMU_OK) {
     e = cudaMemcpyAsync(X, Bp, blk * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream);
     s = (e == cudaSuccess) ? factor_potrs(ctx, L, X, npad, nrhs) : emu_cuda_fail(ctx, e, "refine x0");
   }
   while (s == EMU_OK) {
-    if (digits) {
-      ProfScope ps(ctx, PROF_SOLVE, 2.0 * (double)npad * npad * nrhs, 8.0 * (double)npad * npad);
-      if ((s = symm_digits::multiply(ctx, dp, S, X, nrhs, buf + 4 * blk)) != EMU_OK) break;
-      k_symm_finish<<<4 * ctx->sm_count, 256, 0, ctx->stream>>>(buf + 4 * blk, dp.nz, symm_digits::NR, Bp, R, npad,
-                                                                nrhs);
-      EMU_LAUNCHED(ctx);
-    } else if ((s = symm_residual(ctx, S, X, Bp, R, buf + 4 * blk, nrhs)) != EMU_OK) {
-      break;
-    }
+    if ((s = symm_residual(ctx, S, X, Bp, R, buf + 4 * blk, nrhs)) != EMU_OK) break;
     k_col_norms<<<nrhs, 256, 0, ctx->stream>>>(R, X, Bp, npad, npad, norms);
     ctx->launches++;
     e = cudaGetLastError();
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(hn.data(), norms, 3 * nrhs * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess && digits)
-      e = cudaMemcpyAsync(&hflag, dp.flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) {
       s = emu_cuda_fail(ctx, e, "refine residual");
       break;
-    }
-    if (digits && hflag) {
-      digits = false;  // the same residual on the FP64 pipe, and so from here on
-      continue;
     }
     eta = 0.0;
     for (int c = 0; c < nrhs; c++) {
