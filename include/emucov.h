@@ -28,6 +28,11 @@
  *     emu_create; NULL = the legacy default stream).  Calls that fill an
  *     `info` struct, or that return a status decided on the device
  *     (EMU_ENOTPD, EMU_ETIMEOUT, EMU_ENOCONV), synchronise that stream.
+ *     emu_sample and emu_potrs may return before their device work has ended.
+ *     A bounded wait of theirs that runs out leaves their output unspecified
+ *     and is reported, once, as EMU_ETIMEOUT by the context's next factor,
+ *     empirical covariance, refined solve, batch, emu_sample_host or transform
+ *     in digit form.
  *   - Every call returns an emu_status.  No exception or signal crosses the
  *     ABI.  On EMU_ECUDA the CUDA error string is kept in the context
  *     (emu_last_error).  Arguments are validated on the host before any launch.
@@ -255,6 +260,12 @@ emu_status emu_measure_alu_peaks(emu_ctx *ctx, double *fp64_tflops, double *fp32
  * leave, and the context stays usable.  Synchronises the device.  For tests
  * of failure detection only. */
 emu_status emu_test_wait_hook(emu_ctx *ctx, long long wait_cycles, int withhold_index);
+/* The same for the triangular sweeps of emu_potrs and emu_solve_refine, for
+ * this context only: wait_cycles bounds a wait for a solved slab (<= 0: the
+ * default, about 2 s), and slab withhold_slab (64 rows, counted from the top;
+ * -1 for none) is never published, so that the sweep that waits for it gives
+ * up. */
+emu_status emu_test_sweep_hook(emu_ctx *ctx, long long wait_cycles, int withhold_slab);
 emu_status emu_prof_read(emu_ctx *ctx, int group, int *launches, double *total_ms,
                          double *flops, double *bytes, double *mma_flops);
 

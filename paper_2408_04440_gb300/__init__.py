@@ -34,7 +34,7 @@ MAP_NAMES = ("norm", "dp_sp", "dp_sp_hp", "dp_hp")
 # Every symbol the header declares (checked by the CPU test suite).
 EXPORTED = (
     "emu_create", "emu_destroy", "emu_set_stream", "emu_status_str", "emu_last_error",
-    "emu_launch_count", "emu_host_launch_count", "emu_prof_enable", "emu_prof_read", "emu_prof_timeline", "emu_trace_enable", "emu_trace_read", "emu_potrf_task_list", "emu_test_wait_hook", "emu_schedule", "emu_schedule_info", "emu_measure_alu_peaks", "emu_cov_build", "emu_mat_import",
+    "emu_launch_count", "emu_host_launch_count", "emu_prof_enable", "emu_prof_read", "emu_prof_timeline", "emu_trace_enable", "emu_trace_read", "emu_potrf_task_list", "emu_test_wait_hook", "emu_test_sweep_hook", "emu_schedule", "emu_schedule_info", "emu_measure_alu_peaks", "emu_cov_build", "emu_mat_import",
     "emu_mat_import_host", "emu_cov_from_residuals", "emu_var_recursion", "emu_isht", "emu_sht", "emu_emulate_grid", "emu_cov_build_classfmt",
     "emu_backward_error_est", "emu_mat_clone", "emu_mat_export", "emu_mat_tile_info", "emu_mat_shape",
     "emu_mat_free", "emu_potrf_mp", "emu_sample", "emu_sample_host", "emu_potrs", "emu_solve_refine",
@@ -107,6 +107,7 @@ def load() -> ctypes.CDLL:
     L.emu_prof_enable.argtypes = [vp, i]
     L.emu_trace_enable.argtypes = [vp, i]
     L.emu_test_wait_hook.argtypes = [vp, ctypes.c_longlong, i]
+    L.emu_test_sweep_hook.argtypes = [vp, ctypes.c_longlong, i]
     L.emu_schedule.argtypes = [vp, i, i]
     L.emu_measure_alu_peaks.argtypes = [vp, dpp, dpp]
     L.emu_schedule_info.argtypes = [vp, ctypes.POINTER(i), ctypes.POINTER(i), ctypes.POINTER(i)]
@@ -143,7 +144,7 @@ def load() -> ctypes.CDLL:
     L.emu_batch_release.argtypes = [vp]
     for name in ("emu_create", "emu_destroy", "emu_set_stream", "emu_prof_enable", "emu_prof_read",
                  "emu_trace_enable", "emu_trace_read", "emu_potrf_task_list", "emu_prof_timeline",
-                 "emu_test_wait_hook",
+                 "emu_test_wait_hook", "emu_test_sweep_hook",
                  "emu_schedule", "emu_schedule_info", "emu_measure_alu_peaks",
                  "emu_mat_import_host", "emu_cov_build", "emu_mat_import", "emu_emulate_grid",
                  "emu_cov_build_classfmt", "emu_backward_error_est",
@@ -244,6 +245,10 @@ class Context:
     def test_wait_hook(self, wait_cycles: int = 0, withhold_index: int = -1):
         """Bound of the diagonal POTRF's flag waits (cycles, 0 = default) and one flag index they never see set."""
         self._check(self.lib.emu_test_wait_hook(self.h, int(wait_cycles), int(withhold_index)), "emu_test_wait_hook")
+
+    def test_sweep_hook(self, wait_cycles: int = 0, withhold_slab: int = -1):
+        """Bound of the triangular sweeps' waits (cycles, 0 = default) and one slab that is never published."""
+        self._check(self.lib.emu_test_sweep_hook(self.h, int(wait_cycles), int(withhold_slab)), "emu_test_sweep_hook")
 
     def trace_enable(self, on: bool = True):
         self._check(self.lib.emu_trace_enable(self.h, int(on)), "emu_trace_enable")

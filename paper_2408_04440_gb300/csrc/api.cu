@@ -29,6 +29,13 @@ static emu_status fail_msg(emu_ctx *ctx, emu_status s, const char *msg) {
   return s;
 }
 
+emu_status status_timed_out(emu_ctx *ctx) {
+  const bool own = ctx->h_status[ST_CODE] == DEV_TIMEOUT;
+  if (!own && !ctx->h_status[ST_LATE]) return EMU_OK;
+  EMU_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status + ST_LATE, 0, sizeof(int), ctx->stream));
+  return fail_msg(ctx, EMU_ETIMEOUT, own ? "device wait timed out" : "device wait of an earlier call timed out");
+}
+
 // ------------------------------------------------------------- profiling
 ProfScope::ProfScope(emu_ctx *c, int group, double flops, double bytes, double mma_flops)
     : ctx(c), on(c && c->prof) {
@@ -119,7 +126,7 @@ emu_status emu_create(emu_ctx **out, int device, void *stream) {
   ctx->sm_count = p.multiProcessorCount;
   cudaError_t e = cudaSetDevice(device);
   if (e == cudaSuccess) e = cudaMalloc(&ctx->d_status, ST_WORDS * sizeof(int));
-  if (e == cudaSuccess) e = cudaMallocHost(&ctx->h_status, ST_WORDS * sizeof(int));
+  if (e == cudaSuccess) e = cudaMallocHost(&ctx->h_status, (ST_WORDS + 1) * sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(ctx->d_status, 0, ST_WORDS * sizeof(int));
   if (e == cudaSuccess) e = cudaEventCreate(&ctx->ev0);
   if (e == cudaSuccess) e = cudaEventCreate(&ctx->ev1);
@@ -227,6 +234,13 @@ emu_status emu_test_wait_hook(emu_ctx *ctx, long long wait_cycles, int withhold_
   if (!ctx) return EMU_EINVAL;
   EMU_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
   return set_dag_wait_hook(ctx, wait_cycles, withhold_index);
+}
+
+emu_status emu_test_sweep_hook(emu_ctx *ctx, long long wait_cycles, int withhold_slab) {
+  if (!ctx) return EMU_EINVAL;
+  ctx->sweep_wait = wait_cycles > 0 ? wait_cycles : 0;
+  ctx->sweep_withhold = withhold_slab;
+  return EMU_OK;
 }
 
 emu_status emu_trace_read(emu_ctx *ctx, uint64_t *h_records, size_t max_records, size_t *n_records) {
@@ -421,7 +435,7 @@ emu_status emu_cov_from_residuals(emu_ctx *ctx, const double *dXi, int n, long m
   uint16_t *d_digits = nullptr;
   unsigned long long *d_maxbits = nullptr;
   cudaStream_t st = ctx->stream;
-  cudaError_t e = cudaMemsetAsync(ctx->d_status, 0, ST_WORDS * sizeof(int), st);
+  cudaError_t e = status_clear(ctx);
   if (e == cudaSuccess) e = cudaMallocAsync(&d_items, items.size() * sizeof(gemm64::Item), st);
   if (e == cudaSuccess) e = cudaMallocAsync(&d_segs, segs.size() * sizeof(gemm64::Seg), st);
   if (e == cudaSuccess) e = cudaMallocAsync(&d_exps, (size_t)npad * sizeof(int), st);
@@ -597,8 +611,7 @@ static emu_status collect_status(emu_ctx *ctx, int *pivot) {
   EMU_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
   if (pivot) *pivot = ctx->h_status[ST_PIVOT];
   if (ctx->h_status[ST_CODE] == DEV_NOTPD) return EMU_ENOTPD;
-  if (ctx->h_status[ST_CODE] == DEV_TIMEOUT) return fail_msg(ctx, EMU_ETIMEOUT, "device wait timed out");
-  return EMU_OK;
+  return status_timed_out(ctx);
 }
 
 // Plain FP64 right-looking tile Cholesky on the FP64 pipe, for the tile sizes
@@ -622,7 +635,7 @@ extern "C" emu_status emu_potrf_mp(emu_ctx *ctx, emu_mat *A, const emu_mp_opts *
     return fail_msg(ctx, EMU_EINVAL, "unknown precision map");
   bool mixed = o && (o->eps > 0.0 || o->band != EMU_MAP_NORM);
   EMU_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
-  EMU_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, ST_WORDS * sizeof(int), ctx->stream));
+  EMU_CUDA_TRY(ctx, status_clear(ctx));
   EMU_CUDA_TRY(ctx, cudaEventRecord(ctx->ev0, ctx->stream));
   emu_status s;
   if (A->cs) {
@@ -709,8 +722,10 @@ extern "C" emu_status emu_sample_host(emu_ctx *ctx, const emu_mat *L, int nsampl
     cudaError_t e = cudaMemcpy2DAsync(hY, ldy * sizeof(double), Y, (size_t)L->n * sizeof(double),
                                       (size_t)L->n * sizeof(double), nsamples,
                                       cudaMemcpyDeviceToHost, ctx->stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(ctx->h_status, ctx->d_status, ST_WORDS * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-    if (e != cudaSuccess) s = emu_cuda_fail(ctx, e, "copy Y to host");
+    s = e == cudaSuccess ? status_timed_out(ctx) : emu_cuda_fail(ctx, e, "copy Y to host");
   }
   cudaFreeAsync(Y, ctx->stream);
   cudaStreamSynchronize(ctx->stream);

@@ -791,7 +791,7 @@ emu_status batch_run(emu_ctx *ctx, int count, const emu_cov_params *p, int nb, c
     std::memcpy(B->u, u, sizeof(u));
     if ((s = batch_layout(ctx, B, count, p, nb)) != EMU_OK) return s;
   }
-  EMU_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, ST_WORDS * sizeof(int), ctx->stream));
+  EMU_CUDA_TRY(ctx, status_clear(ctx));
   // covariances, tile norms and the precision map of every matrix
   if ((s = launch_cov_build_batch(ctx, B->d_inst, count, B->maxL, B->ntab, B->d_tile_inst, B->ntiles, nb, B->tables,
                                   B->t64, B->partial)) != EMU_OK)
@@ -886,10 +886,7 @@ emu_status batch_run(emu_ctx *ctx, int count, const emu_cov_params *p, int nb, c
       f.ms = ms;
     }
   }
-  if (code == DEV_TIMEOUT) {
-    ctx->last_error = "device wait timed out";
-    return EMU_ETIMEOUT;
-  }
+  if ((s = status_timed_out(ctx)) != EMU_OK) return s;
   if (nbad > 0 || code == DEV_NOTPD) {
     ctx->last_error = "covariances of the batch are not positive definite (see their info.pivot; the others are complete)";
     return EMU_ENOTPD;

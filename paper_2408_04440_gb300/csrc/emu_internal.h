@@ -30,9 +30,16 @@ __host__ __device__ inline void tile_coords(long t, int NT, int *i, int *j) {
 }
 inline long tile_count(int NT) { return (long)NT * (NT + 1) / 2; }
 
-// Device status word written by kernels and read back at sync points.
-enum { ST_CODE = 0, ST_PIVOT = 1, ST_AUX = 2, ST_WORDS = 4 };
+// Device status word written by kernels and read back at sync points.  Calls
+// clear the words before ST_LATE when they begin.  ST_LATE stays: it records
+// that a wait ran out, also in a call that returns before its device work ends
+// (emu_potrs, emu_sample), until a call that reads the status reports it.
+enum { ST_CODE = 0, ST_PIVOT = 1, ST_AUX = 2, ST_LATE = 3, ST_WORDS = 4 };
 enum { DEV_OK = 0, DEV_NOTPD = 1, DEV_TIMEOUT = 2 };
+__device__ inline void status_timeout(int *st, int aux) {
+  if (atomicCAS(&st[ST_CODE], DEV_OK, DEV_TIMEOUT) == DEV_OK) st[ST_AUX] = aux;
+  st[ST_LATE] = 1;
+}
 
 // Matrix states.
 enum { MAT_COV = 0, MAT_FACTOR64 = 1, MAT_FACTOR_MIXED = 2 };
@@ -57,7 +64,7 @@ struct emu_ctx {
   cudaStream_t stream = nullptr;
   int sm_count = 0;
   int *d_status = nullptr;    // ST_WORDS ints
-  int *h_status = nullptr;    // pinned mirror
+  int *h_status = nullptr;    // pinned mirror, and one more word for a call's own flag
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   uint64_t launches = 0;       // kernels of this library, graph nodes included
   uint64_t host_launches = 0;  // launch calls the host made (a graph replay counts once)
@@ -96,6 +103,10 @@ struct emu_ctx {
   void *batch = nullptr;
   // single-matrix mixed factor (mixed.cu): captured graph, tuning table
   void *mixed = nullptr;
+  // test hook of the triangular sweeps: wait bound in cycles (0: default) and
+  // the slab that is never published (-1: none)
+  long long sweep_wait = 0;
+  int sweep_withhold = -1;
   // optional device-side task trace of the dataflow POTRF
   bool trace_on = false;
   unsigned long long *trace_buf = nullptr;
@@ -176,6 +187,13 @@ emu_status emu_cuda_fail(emu_ctx *ctx, cudaError_t e, const char *what);
     cudaError_t _e = (expr);                                      \
     if (_e != cudaSuccess) return emu_cuda_fail((ctx), _e, #expr); \
   } while (0)
+// The status words a call clears when it begins.
+inline cudaError_t status_clear(emu_ctx *ctx) {
+  return cudaMemsetAsync(ctx->d_status, 0, ST_LATE * sizeof(int), ctx->stream);
+}
+// EMU_ETIMEOUT when the mirror of the status, read and waited for, says that a
+// wait ran out in this call or in an earlier one that did not report it.
+emu_status status_timed_out(emu_ctx *ctx);
 // After a launch: count it and surface launch-configuration errors.
 #define EMU_LAUNCHED(ctx)                                                   \
   do {                                                                      \

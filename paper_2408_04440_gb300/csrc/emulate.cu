@@ -480,7 +480,7 @@ emu_status emu_var_recursion(emu_ctx *ctx, const double *dXi, int n, int T, long
   if (!ctx || !dXi || !dF || n < 1 || T < 1 || ldxi < n || ldf < n || P < 0 || P > kMaxP || (P > 0 && !dPhi))
     return EMU_EINVAL;
   EMU_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
-  EMU_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, ST_WORDS * sizeof(int), ctx->stream));
+  EMU_CUDA_TRY(ctx, status_clear(ctx));
   auto var = P == 1 ? k_var<1> : P == 2 ? k_var<2> : P == 3 ? k_var<3> : P == 4 ? k_var<4> : k_var<kMaxP>;
   var<<<(n + 31) / 32, 32, 0, ctx->stream>>>(dXi, ldxi, n, T, dPhi, P, dF, ldf, ctx->d_status);
   EMU_LAUNCHED(ctx);
@@ -494,7 +494,7 @@ emu_status emu_isht(emu_ctx *ctx, const double *dF, int L, int T, long ldf, int 
       ldz < (long)ntheta * nphi)
     return EMU_EINVAL;
   EMU_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
-  EMU_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, ST_WORDS * sizeof(int), ctx->stream));
+  EMU_CUDA_TRY(ctx, status_clear(ctx));
   const double flops = 2.0 * (double)L * L * ntheta * T + 4.0 * (double)L * ntheta * nphi * T;
   if (by_digits(L, flops) && nphi <= 65535) {
     ProfScope ps(ctx, PROF_SOLVE, flops, 0.0);
@@ -513,7 +513,7 @@ emu_status emu_sht(emu_ctx *ctx, const double *dZ, int ntheta, int nphi, int T, 
   const size_t Q = 2 * (size_t)L - 1;
   if ((4 * Q + ntheta) * sizeof(double) > 48 * 1024 || nphi * sizeof(double) > 48 * 1024) return EMU_EINVAL;
   EMU_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
-  EMU_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, ST_WORDS * sizeof(int), ctx->stream));
+  EMU_CUDA_TRY(ctx, status_clear(ctx));
   const double flops = 4.0 * (double)L * ntheta * nphi * T + 4.0 * (double)L * Q * ntheta * T;
   if (by_digits(L, flops)) {
     ProfScope ps(ctx, PROF_SOLVE, flops, 0.0);

@@ -218,7 +218,7 @@ emu_status sample64_digits(emu_ctx *ctx, const emu_mat *L, const double *Z, long
   int *ae = reinterpret_cast<int *>(b + o_ae), *ze = reinterpret_cast<int *>(b + o_ze);
   CUtensorMap ma, mz;
   // an earlier factor's failure must not stop the draws of this one
-  if (cudaMemsetAsync(ctx->d_status, 0, ST_WORDS * sizeof(int), ctx->stream) != cudaSuccess) st = EMU_ECUDA;
+  if (status_clear(ctx) != cudaSuccess) st = EMU_ECUDA;
   if (st == EMU_OK) st = gemm64::make_map(ctx, &ma, ad, npad, (uint64_t)gemm64::NS * grows, gemm64::BM);
   if (st == EMU_OK) st = gemm64::make_map(ctx, &mz, zd, npad, (uint64_t)gemm64::NS * s_pad, gemm64::BN);
   if (st == EMU_OK) st = gemm64::launch_slice_cols(ctx, Z, ldz, s, s_pad, (int)npad, ze, zd);

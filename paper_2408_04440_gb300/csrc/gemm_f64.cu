@@ -66,7 +66,7 @@ __device__ inline bool failed(const int *st) { return *((volatile const int *)st
 
 __device__ inline void raise_timeout(Shared *sh, int *status) {
   sh->abort = 1;
-  if (atomicCAS(&status[ST_CODE], DEV_OK, DEV_TIMEOUT) == DEV_OK) status[ST_AUX] = 4;
+  status_timeout(status, 4);
 }
 
 // ------------------------------------------------------------- digits

@@ -75,7 +75,7 @@ static_assert(sizeof(Shared) <= BAR_BYTES, "barrier block");
 
 __device__ inline void raise_timeout(Shared *sh, int *status) {
   sh->abort = 1;
-  if (atomicCAS(&status[ST_CODE], DEV_OK, DEV_TIMEOUT) == DEV_OK) status[ST_AUX] = 1;
+  status_timeout(status, 1);
 }
 
 __global__ void __launch_bounds__(NTHREADS, 1)

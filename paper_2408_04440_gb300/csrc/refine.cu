@@ -205,11 +205,12 @@ emu_status refine_solve(emu_ctx *ctx, const emu_mat *L, const emu_mat *S, const 
     e = cudaGetLastError();
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(hn.data(), norms, 3 * nrhs * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(ctx->h_status, ctx->d_status, ST_WORDS * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-    if (e != cudaSuccess) {
-      s = emu_cuda_fail(ctx, e, "refine residual");
-      break;
-    }
+    // a sweep that gave up has left X or its correction half solved
+    s = e == cudaSuccess ? status_timed_out(ctx) : emu_cuda_fail(ctx, e, "refine residual");
+    if (s != EMU_OK) break;
     eta = 0.0;
     for (int c = 0; c < nrhs; c++) {
       double den = frobS * sqrt(hn[3 * c + 1]) + sqrt(hn[3 * c + 2]);

@@ -420,19 +420,16 @@ emu_status sht_passes(emu_ctx *ctx, const double *dZ, int ntheta, int nphi, int 
 emu_status finish(emu_ctx *ctx, char *blob, const int *flag, emu_status s) {
   cudaError_t e = cudaSuccess;
   if (s == EMU_OK) {
-    e = cudaMemcpyAsync(ctx->h_status, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
+    e = cudaMemcpyAsync(ctx->h_status, ctx->d_status, ST_WORDS * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(ctx->h_status + 3, flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
+      e = cudaMemcpyAsync(ctx->h_status + ST_WORDS, flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
   }
   cudaFreeAsync(blob, ctx->stream);
   if (s != EMU_OK) return s;
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) return emu_cuda_fail(ctx, e, "transform");
-  if (ctx->h_status[ST_CODE] == DEV_TIMEOUT) {
-    ctx->last_error = "device wait timed out";
-    return EMU_ETIMEOUT;
-  }
-  return ctx->h_status[3] ? EMU_ESTATE : EMU_OK;
+  s = status_timed_out(ctx);
+  return s != EMU_OK ? s : ctx->h_status[ST_WORDS] ? EMU_ESTATE : EMU_OK;
 }
 
 }  // namespace

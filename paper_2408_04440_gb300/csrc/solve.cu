@@ -33,7 +33,7 @@ namespace {
 constexpr int SL = 64;    // rows of a slab
 constexpr int LDA = 68;   // FP32 columns of a block in shared memory: 16-byte aligned, float4 reads down a column
 constexpr int LDD = 66;   // FP64 columns
-// wait bound in SM clock cycles (about 2 s at 2 GHz)
+// default wait bound in SM clock cycles (about 2 s at 2 GHz)
 constexpr long long kSweepWaitCycles = 4000000000ll;
 
 __device__ inline bool failed(const int *st) { return *((volatile const int *)st) != DEV_OK; }
@@ -70,11 +70,13 @@ __device__ inline double from_words(const unsigned long long (&w)[2]) {
 // X <- L^{-1} X or (BACK) X <- L^{-T} X.  ticket: the next slab per group, zero
 // before the launch.  xs: the solved slabs, [group][slab][64][P] tagged values,
 // zero before the launch.  cls null: every tile is FP64 (plain factor).
+// wait_cycles: bound of a wait; withhold: slab that is not published (for
+// tests; else -1).
 template <typename F, int P, bool BACK>
 __global__ void __launch_bounds__(256, sizeof(F) == 4 ? 2 : 1)
     k_sweep(const double *__restrict__ t64, const float *__restrict__ t32, const unsigned char *__restrict__ cls, int nb,
             int NT, int nslab, double *__restrict__ X, long ld, int nrhs, unsigned long long *__restrict__ xs,
-            int *__restrict__ ticket, int *st) {
+            int *__restrict__ ticket, int *st, long long wait_cycles, int withhold) {
   constexpr int NQ = P / 4;                       // right-hand sides per thread
   constexpr int NW = sizeof(F) / 4;               // words per published value
   constexpr int LD = sizeof(F) == 4 ? LDA : LDD;  // block column stride
@@ -194,10 +196,9 @@ __global__ void __launch_bounds__(256, sizeof(F) == 4 ? 2 : 1)
         }
         if (tid == 0) {
           if (j + 1 < k)
-            while (get_word(xo + (size_t)(P - 1) * NW) < kTag && !failed(st) && clock64() - t0 <= kSweepWaitCycles)
+            while (get_word(xo + (size_t)(P - 1) * NW) < kTag && !failed(st) && clock64() - t0 <= wait_cycles)
               __nanosleep(256);
-          if (clock64() - t0 > kSweepWaitCycles && atomicCAS(&st[ST_CODE], DEV_OK, DEV_TIMEOUT) == DEV_OK)
-            st[ST_AUX] = 6;
+          if (clock64() - t0 > wait_cycles) status_timeout(st, 6);
         }
         if (__syncthreads_or(tid == 0 && failed(st))) {
           bad = true;
@@ -328,8 +329,10 @@ __global__ void __launch_bounds__(256, sizeof(F) == 4 ? 2 : 1)
 #pragma unroll
       for (int r = 0; r < NR; r++) {
         const int c = w + 8 * r;
-        publish(xo + ((size_t)lane * P + c) * NW, y0[r]);
-        publish(xo + ((size_t)(lane + 32) * P + c) * NW, y1[r]);
+        if (s != withhold) {
+          publish(xo + ((size_t)lane * P + c) * NW, y0[r]);
+          publish(xo + ((size_t)(lane + 32) * P + c) * NW, y1[r]);
+        }
         if (c < p) {
           X[(size_t)s * SL + lane + (size_t)(c0 + c) * ld] = (double)y0[r];
           X[(size_t)s * SL + lane + 32 + (size_t)(c0 + c) * ld] = (double)y1[r];
@@ -355,11 +358,14 @@ emu_status sweeps(emu_ctx *ctx, const emu_mat *L, double *X, long ldx, int nrhs)
   cudaError_t e = cudaMemsetAsync(ws, 0, 2 * words * sizeof(*ws), ctx->stream);
   const unsigned char *cls = L->state == MAT_FACTOR64 ? nullptr : L->d_cls;
   const dim3 grid((unsigned)std::min(nslab, (sizeof(F) == 4 ? 2 : 1) * ctx->sm_count), (unsigned)groups);
+  const long long wait = ctx->sweep_wait > 0 ? ctx->sweep_wait : kSweepWaitCycles;
   if (e == cudaSuccess) {
     k_sweep<F, P, false><<<grid, 256, smem, ctx->stream>>>(L->t64, L->t32, cls, nb, NT, nslab, X, ldx, nrhs, ws,
-                                                           reinterpret_cast<int *>(ws + xw), ctx->d_status);
+                                                           reinterpret_cast<int *>(ws + xw), ctx->d_status, wait,
+                                                           ctx->sweep_withhold);
     k_sweep<F, P, true><<<grid, 256, smem, ctx->stream>>>(L->t64, L->t32, cls, nb, NT, nslab, X, ldx, nrhs, ws + words,
-                                                          reinterpret_cast<int *>(ws + words + xw), ctx->d_status);
+                                                          reinterpret_cast<int *>(ws + words + xw), ctx->d_status, wait,
+                                                          ctx->sweep_withhold);
     ctx->launches += 2;
     ctx->host_launches += 2;
     e = cudaGetLastError();
@@ -373,7 +379,7 @@ emu_status sweeps(emu_ctx *ctx, const emu_mat *L, double *X, long ldx, int nrhs)
 emu_status factor_potrs(emu_ctx *ctx, const emu_mat *L, double *X, long ldx, int nrhs) {
   ProfScope ps(ctx, PROF_SOLVE, 2.0 * (double)L->n * L->n * nrhs, 4.0 * (double)L->n * L->n);
   // an earlier factor's failure must not stop the solves with this one
-  EMU_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, ST_WORDS * sizeof(int), ctx->stream));
+  EMU_CUDA_TRY(ctx, status_clear(ctx));
   if (L->state == MAT_FACTOR64)
     return nrhs <= 4 ? sweeps<double, 4>(ctx, L, X, ldx, nrhs) : sweeps<double, 16>(ctx, L, X, ldx, nrhs);
   return nrhs <= 4    ? sweeps<float, 4>(ctx, L, X, ldx, nrhs)
