@@ -688,6 +688,8 @@ extern "C" emu_status emu_sample(emu_ctx *ctx, const emu_mat *L, int nsamples, u
   EMU_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
   long npad = (long)L->nt * L->nb;
   double *Z = nullptr;
+  // an earlier factor's failure must not stop the draws of this one
+  EMU_CUDA_TRY(ctx, status_clear(ctx));
   EMU_CUDA_TRY(ctx, cudaMallocAsync(&Z, (size_t)npad * nsamples * sizeof(double), ctx->stream));
   emu_status s = launch_normals(ctx, seed, stream_id, (int)npad, nsamples, Z, npad);
   if (s == EMU_OK) {

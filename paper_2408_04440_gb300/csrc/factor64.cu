@@ -217,9 +217,7 @@ emu_status sample64_digits(emu_ctx *ctx, const emu_mat *L, const double *Z, long
   uint16_t *ad = reinterpret_cast<uint16_t *>(b + o_a), *zd = reinterpret_cast<uint16_t *>(b + o_z);
   int *ae = reinterpret_cast<int *>(b + o_ae), *ze = reinterpret_cast<int *>(b + o_ze);
   CUtensorMap ma, mz;
-  // an earlier factor's failure must not stop the draws of this one
-  if (status_clear(ctx) != cudaSuccess) st = EMU_ECUDA;
-  if (st == EMU_OK) st = gemm64::make_map(ctx, &ma, ad, npad, (uint64_t)gemm64::NS * grows, gemm64::BM);
+  st = gemm64::make_map(ctx, &ma, ad, npad, (uint64_t)gemm64::NS * grows, gemm64::BM);
   if (st == EMU_OK) st = gemm64::make_map(ctx, &mz, zd, npad, (uint64_t)gemm64::NS * s_pad, gemm64::BN);
   if (st == EMU_OK) st = gemm64::launch_slice_cols(ctx, Z, ldz, s, s_pad, (int)npad, ze, zd);
   for (int i0 = 0; i0 < NT && st == EMU_OK; i0 += g) {
