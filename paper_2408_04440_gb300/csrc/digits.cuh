@@ -33,7 +33,7 @@ __device__ inline long long to_fixed(double x, int e) {
   unsigned long long m = b & 0xfffffffffffffull;
   if (ex > 0) m |= 1ull << 52;
   else ex = 1;
-  const int sh = ex - 1019 - e;  // x 2^(56 - e) = m 2^sh, sh <= 3
+  const int sh = ex - 1019 - e;  // x 2^(56 - e) = m 2^sh, sh <= 3 (<= 6 and m < 2^50 for denormal rows)
   unsigned long long X;
   if (sh >= 0) {
     X = m << sh;

@@ -56,11 +56,12 @@ emu_status make_map(emu_ctx *ctx, CUtensorMap *map, const void *base, uint64_t i
                     uint32_t box_rows);
 
 // Exponent arrays hold e + kExpBias, so that a zeroed array (cudaMemset 0)
-// holds the lowest exponent; readers clamp e at kExpMin, which only rows of
-// zeros reach.  A row with an infinity or a NaN holds kExpPoison: its digits
+// holds the lowest exponent; readers clamp e at kExpMin.  A row below 2^kExpMin
+// loses nothing by that: the last digit's unit is then 2^-1080, below FP64's
+// smallest number.  A row with an infinity or a NaN holds kExpPoison: its digits
 // are zeros and every product with it is NaN, as in floating point.
 constexpr int kExpBias = 1024;
-constexpr int kExpMin = -960;
+constexpr int kExpMin = -kExpBias;
 constexpr int kExpPoison = 1 << 20;
 
 // Row exponents of listed tiles: jobs {tile, -, exponent base}; a tile is read
