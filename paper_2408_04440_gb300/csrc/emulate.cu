@@ -496,7 +496,7 @@ emu_status emu_isht(emu_ctx *ctx, const double *dF, int L, int T, long ldf, int 
   EMU_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
   EMU_CUDA_TRY(ctx, status_clear(ctx));
   const double flops = 2.0 * (double)L * L * ntheta * T + 4.0 * (double)L * ntheta * nphi * T;
-  if (by_digits(L, flops) && nphi <= 65535) {
+  if (by_digits(L, flops)) {
     ProfScope ps(ctx, PROF_SOLVE, flops, 0.0);
     const emu_status s = isht_digits(ctx, dF, L, T, ldf, ntheta, nphi, dZ, ldz);
     if (s != EMU_ENOMEM && s != EMU_ESTATE) return s;

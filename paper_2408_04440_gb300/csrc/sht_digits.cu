@@ -439,6 +439,8 @@ emu_status isht_digits(emu_ctx *ctx, const double *dF, int L, int T, long ldf, i
   const size_t npair = (size_t)L * (L + 1) / 2, Lp = pad(L, 32), Kq = pad(2L * L, 32), cpad = pad(ntheta, gemm64::BN),
                npj = pad(nphi, gemm64::BN);
   const double ktot_d = 16.0 * Lp * (Lp + 32.0) / 32.0;  // sum over orders of order_k
+  // rings in blocks of 32, and longitudes, count on the second axis of a grid
+  if (ntheta > 32 * 65535 || nphi > 65535) return EMU_ENOMEM;
   if (npair * ntheta > (size_t)1 << 31 || 32.0 * ktot_d > 2147483647.0) return EMU_ENOMEM;
   const size_t ktot = (size_t)gemm64::order_koff(L, (int)Lp - 32) + 32 * 32;
   const int Tc = steps_per_pass(T, 2.0 * NS * ((double)ntheta * Kq + 2.0 * ktot) + 16.0 * L * ntheta);

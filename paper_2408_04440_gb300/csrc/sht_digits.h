@@ -1,6 +1,7 @@
 // sht_digits.h -- the spherical-harmonic transforms as digit products on the
 // tensor cores (sht_digits.cu).  Both wait for the result and return
-//   EMU_ENOMEM  the workspace does not fit: nothing was written;
+//   EMU_ENOMEM  the workspace does not fit, or the sizes do not: nothing was
+//               written;
 //   EMU_ESTATE  an operand held an infinity or a NaN: the caller runs the
 //               direct sums, which carry them as floating point does.
 // d_status is zero on entry.
