@@ -18,7 +18,8 @@ namespace {
 // (i, j) for j <= i, tile (j, i) read transposed for j > i), operands staged
 // through shared memory in 32-wide K chunks so that every global read is
 // coalesced.  part[z][row][P] of range z and group blockIdx.z; deterministic:
-// one CTA owns each partial sum, k_symm_finish adds the ranges in order.
+// one CTA owns each partial sum, k_symm_finish adds the ranges in order.  With
+// one range (from 58000 rows times groups on) R = Bm - S X is written here.
 //
 // Bound by FP64 issue from a few right-hand sides on.  As digit products on the
 // tensor cores n = 16384 with 16 columns takes 1.5 ms instead of 7.3, but that
@@ -28,8 +29,8 @@ namespace {
 constexpr int RK = 32;
 template <int P>
 __global__ void __launch_bounds__(256)
-    k_symm_part(const double *__restrict__ t64, int nb, int NT, const double *__restrict__ X, double *__restrict__ part,
-                long npad, int nrhs) {
+    k_symm_part(const double *__restrict__ t64, int nb, int NT, const double *__restrict__ X,
+                const double *__restrict__ Bm, double *__restrict__ R, double *__restrict__ part, long npad, int nrhs) {
   constexpr int KG = P == 1 ? 4 : 1;       // thread groups that share the K chunk
   constexpr int NQ = P == 1 ? 1 : P / 4;   // right-hand sides per thread
   __shared__ double a[RK][RS + 1];
@@ -79,13 +80,22 @@ __global__ void __launch_bounds__(256)
       __syncthreads();
     }
   }
-  double *o = part + (((size_t)blockIdx.z * gridDim.y + blockIdx.y) * npad + g0 + mm) * P;
   if (KG == 4) {
     double *red = &a[0][0];
     red[tid] = acc[0];
     __syncthreads();
-    if (tid < RS) o[0] = (red[tid] + red[tid + 64]) + (red[tid + 128] + red[tid + 192]);
+    if (tid >= RS) return;
+    acc[0] = (red[tid] + red[tid + 64]) + (red[tid + 128] + red[tid + 192]);
+  }
+  if (gridDim.y == 1) {
+    // one range: the product is complete
+#pragma unroll
+    for (int w = 0; w < NQ; w++) {
+      const size_t o = (size_t)(g0 + mm) + (size_t)(c0 + q0 + 4 * w) * npad;
+      if (q0 + 4 * w < p) R[o] = Bm[o] - acc[w];
+    }
   } else {
+    double *o = part + (((size_t)blockIdx.z * gridDim.y + blockIdx.y) * npad + g0 + mm) * P;
 #pragma unroll
     for (int w = 0; w < NQ; w++) o[q0 + 4 * w] = acc[w];
   }
@@ -148,7 +158,7 @@ __global__ void k_axpy(double *__restrict__ X, const double *__restrict__ D, lon
 
 }  // namespace
 
-// R = B - S X (npad x nrhs each); part: groups nz npad P doubles.
+// R = B - S X (npad x nrhs each); part: the split's partial sums.
 static emu_status symm_residual(emu_ctx *ctx, const emu_mat *S, const double *X, const double *Bp, double *R,
                                 double *part, int nrhs) {
   const long npad = (long)S->nt * S->nb;
@@ -160,8 +170,9 @@ static emu_status symm_residual(emu_ctx *ctx, const emu_mat *S, const double *X,
               : sh.P == 8  ? k_symm_part<8>
               : sh.P == 16 ? k_symm_part<16>
                            : k_symm_part<32>;
-  kern<<<grid, 256, 0, ctx->stream>>>(S->t64, S->nb, S->nt, X, part, npad, nrhs);
+  kern<<<grid, 256, 0, ctx->stream>>>(S->t64, S->nb, S->nt, X, Bp, R, part, npad, nrhs);
   EMU_LAUNCHED(ctx);
+  if (sh.nz == 1) return EMU_OK;
   k_symm_finish<<<4 * ctx->sm_count, 256, 0, ctx->stream>>>(part, sh.nz, sh.P, Bp, R, npad, nrhs);
   EMU_LAUNCHED(ctx);
   return EMU_OK;
@@ -176,8 +187,7 @@ emu_status refine_solve(emu_ctx *ctx, const emu_mat *L, const emu_mat *S, const 
   size_t blk = (size_t)npad * nrhs;
   double *buf = nullptr, *norms = nullptr;
   const ResidualSplit sh = residual_split(ctx->sm_count, S->nt, S->nb, nrhs);
-  const size_t part = (size_t)sh.groups * sh.nz * npad * sh.P;
-  EMU_CUDA_TRY(ctx, cudaMallocAsync(&buf, (4 * blk + part) * sizeof(double), ctx->stream));
+  EMU_CUDA_TRY(ctx, cudaMallocAsync(&buf, (4 * blk + sh.partial(npad)) * sizeof(double), ctx->stream));
   EMU_CUDA_TRY(ctx, cudaMallocAsync(&norms, 3 * nrhs * sizeof(double), ctx->stream));
   double *Bp = buf, *X = buf + blk, *R = buf + 2 * blk, *D = buf + 3 * blk;
   std::vector<double> hn(3 * nrhs);

@@ -35,6 +35,10 @@ constexpr int LDA = 68;   // FP32 columns of a block in shared memory: 16-byte a
 constexpr int LDD = 66;   // FP64 columns
 // default wait bound in SM clock cycles (about 2 s at 2 GHz)
 constexpr long long kSweepWaitCycles = 4000000000ll;
+// Published values of the groups of one launch: 16 bytes per FP32 entry of X in
+// both sweeps, 32 per FP64 one.  64 MB of them are 2000 slabs, several times the
+// CTAs that are resident; one group takes more from n = 130000 on.
+constexpr size_t kSweepWorkspace = (size_t)64 << 20;
 
 __device__ inline bool failed(const int *st) { return *((volatile const int *)st) != DEV_OK; }
 
@@ -351,21 +355,35 @@ emu_status sweeps(emu_ctx *ctx, const emu_mat *L, double *X, long ldx, int nrhs)
   static std::atomic<uint64_t> attr_f{0}, attr_b{0};
   EMU_CUDA_TRY(ctx, smem_limit_once(attr_f, ctx->device, (const void *)k_sweep<F, P, false>, smem));
   EMU_CUDA_TRY(ctx, smem_limit_once(attr_b, ctx->device, (const void *)k_sweep<F, P, true>, smem));
-  // per sweep: the tagged values, then the groups' tickets; all zero
-  const size_t xw = (size_t)groups * nslab * SL * P * (sizeof(F) / 4), words = xw + ((size_t)groups + 1) / 2;
+  // per sweep: a group's tagged values and, in one more word, its ticket; all
+  // zero.  As many groups at a time as the workspace holds, fewer where the
+  // device does not have that much.
+  const size_t gw = (size_t)nslab * SL * P * (sizeof(F) / 4), unit = 2 * (gw + 1) * sizeof(unsigned long long);
+  int some = (int)std::max<size_t>(1, std::min<size_t>(groups, kSweepWorkspace / unit));
   unsigned long long *ws = nullptr;
-  EMU_CUDA_TRY(ctx, cudaMallocAsync(&ws, 2 * words * sizeof(*ws), ctx->stream));
-  cudaError_t e = cudaMemsetAsync(ws, 0, 2 * words * sizeof(*ws), ctx->stream);
+  cudaError_t e = cudaMallocAsync(&ws, some * unit, ctx->stream);
+  while (e == cudaErrorMemoryAllocation && some > 1) {
+    cudaGetLastError();
+    some = (some + 1) / 2;
+    e = cudaMallocAsync(&ws, some * unit, ctx->stream);
+  }
+  if (e != cudaSuccess) return emu_cuda_fail(ctx, e, "triangular sweeps");
+  const size_t xw = some * gw, words = some * (gw + 1);
   const unsigned char *cls = L->state == MAT_FACTOR64 ? nullptr : L->d_cls;
-  const dim3 grid((unsigned)std::min(nslab, (sizeof(F) == 4 ? 2 : 1) * ctx->sm_count), (unsigned)groups);
   const long long wait = ctx->sweep_wait > 0 ? ctx->sweep_wait : kSweepWaitCycles;
-  if (e == cudaSuccess) {
-    k_sweep<F, P, false><<<grid, 256, smem, ctx->stream>>>(L->t64, L->t32, cls, nb, NT, nslab, X, ldx, nrhs, ws,
+  for (int g = 0; g < groups && e == cudaSuccess; g += some) {
+    const dim3 grid((unsigned)std::min(nslab, (sizeof(F) == 4 ? 2 : 1) * ctx->sm_count),
+                    (unsigned)std::min(some, groups - g));
+    double *Xg = X + (size_t)g * P * ldx;
+    const int left = nrhs - g * P;
+    e = cudaMemsetAsync(ws, 0, some * unit, ctx->stream);
+    if (e != cudaSuccess) break;
+    k_sweep<F, P, false><<<grid, 256, smem, ctx->stream>>>(L->t64, L->t32, cls, nb, NT, nslab, Xg, ldx, left, ws,
                                                            reinterpret_cast<int *>(ws + xw), ctx->d_status, wait,
                                                            ctx->sweep_withhold);
-    k_sweep<F, P, true><<<grid, 256, smem, ctx->stream>>>(L->t64, L->t32, cls, nb, NT, nslab, X, ldx, nrhs, ws + words,
-                                                          reinterpret_cast<int *>(ws + words + xw), ctx->d_status, wait,
-                                                          ctx->sweep_withhold);
+    k_sweep<F, P, true><<<grid, 256, smem, ctx->stream>>>(L->t64, L->t32, cls, nb, NT, nslab, Xg, ldx, left,
+                                                          ws + words, reinterpret_cast<int *>(ws + words + xw),
+                                                          ctx->d_status, wait, ctx->sweep_withhold);
     ctx->launches += 2;
     ctx->host_launches += 2;
     e = cudaGetLastError();

@@ -1,7 +1,7 @@
 """The split of the refinement residual over the chip (refine_split.h, host arithmetic): every tile size, tile count and
 number of right-hand sides that a matrix can have, one 64-wide tile included, gives a group width, groups that hold the
-right-hand sides and at least one and at most as many column ranges as there are tile columns.  A division by a count that
-is zero for the smallest sizes ends the process here."""
+right-hand sides, at least one and at most as many column ranges as there are tile columns, and partial sums of at most 30
+MB.  A division by a count that is zero for the smallest sizes ends the process here."""
 import os
 import subprocess
 
@@ -18,7 +18,8 @@ int main() {
         for (int sm : {1, 148, 152}) {
           const ResidualSplit s = residual_split(sm, nt, nb, nrhs);
           const bool width = s.P == 1 || s.P == 4 || s.P == 8 || s.P == 16 || s.P == 32;
-          if (!width || (long)s.groups * s.P < nrhs || (long)(s.groups - 1) * s.P >= nrhs || s.nz < 1 || s.nz > nt) {
+          if (!width || (long)s.groups * s.P < nrhs || (long)(s.groups - 1) * s.P >= nrhs || s.nz < 1 || s.nz > nt ||
+              s.partial((long)nt * nb) > 12ul * 64 * 32 * sm) {
             std::printf("nb %d nt %d nrhs %d sm %d: P %d groups %d nz %d\\n", nb, nt, nrhs, sm, s.P, s.groups, s.nz);
             return 1;
           }
