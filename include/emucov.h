@@ -242,6 +242,18 @@ emu_status emu_schedule(emu_ctx *ctx, int use_graphs, int tuning);
  * factor. */
 emu_status emu_schedule_info(emu_ctx *ctx, int *tried, int *reserved, int *reserved_fp64);
 
+/* on != 0: the plain FP64 factor (emu_potrf_mp without eps), its draws and the
+ * spherical-harmonic transforms of this context form all their sums in FP64
+ * arithmetic; off by default.  By default they take, from certain sizes on,
+ * exact products of the operands' digits on the tensor cores, 56 bits of every
+ * entry below the largest of its row: as accurate as FP64 arithmetic relative
+ * to those largest entries, and many times faster (n = 10000: 24 ms instead of
+ * 331), but entries far below them are not as accurate relative to themselves,
+ * and where the digits do not fit the device's free memory a call forms its sums
+ * in FP64 arithmetic, with other last bits.  For cross-checks, for results whose
+ * small entries matter, and for bits that do not depend on free memory. */
+emu_status emu_fp64_arithmetic(emu_ctx *ctx, int on);
+
 /* Measured FMA rates of the context's device, in TFLOP/s (2 flops per FMA):
  * eight independent FP64 (FP32) FMA chains per thread, eight CTAs of 256
  * threads per SM, timed with CUDA events; the denominators of the rooflines of
@@ -426,11 +438,13 @@ emu_status emu_mat_free(emu_mat *A);
 
 /* ------------------------------------------------------------------ factor */
 /* Factor A = L L^T in place (A must hold a covariance, state 0).  Plain FP64
- * when o == NULL or o->eps <= 0 (with nb a multiple of 128 the trailing updates
- * and block products are formed on the tensor cores with FP64 accuracy, exact
- * digit products rounded once; where their workspace does not fit, and for
- * other nb, in FP64 arithmetic), otherwise the adaptive mixed-precision tile
- * factor described at emu_mp_opts.  On a non-positive pivot returns
+ * when o == NULL or o->eps <= 0, otherwise the adaptive mixed-precision tile
+ * factor described at emu_mp_opts.  With nb a multiple of 128 the plain FP64
+ * factor forms its trailing updates and block products as digit products (see
+ * emu_fp64_arithmetic): its error meets the scaled bound of a factor formed in
+ * FP64 arithmetic, |L L^T - A|_ij <= c n 2^-53 sqrt(A_ii A_jj), entry by entry.
+ * Other nb, and a workspace that does not fit, run in FP64 arithmetic, whose
+ * bound is c n 2^-53 (|L| |L|^T)_ij.  On a non-positive pivot returns
  * EMU_ENOTPD with info->pivot set and leaves A in an unspecified state. */
 emu_status emu_potrf_mp(emu_ctx *ctx, emu_mat *A, const emu_mp_opts *o,
                         emu_factor_info *info);

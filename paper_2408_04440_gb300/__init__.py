@@ -34,7 +34,7 @@ MAP_NAMES = ("norm", "dp_sp", "dp_sp_hp", "dp_hp")
 # Every symbol the header declares (checked by the CPU test suite).
 EXPORTED = (
     "emu_create", "emu_destroy", "emu_set_stream", "emu_status_str", "emu_last_error",
-    "emu_launch_count", "emu_host_launch_count", "emu_prof_enable", "emu_prof_read", "emu_prof_timeline", "emu_trace_enable", "emu_trace_read", "emu_potrf_task_list", "emu_test_wait_hook", "emu_test_sweep_hook", "emu_schedule", "emu_schedule_info", "emu_measure_alu_peaks", "emu_cov_build", "emu_mat_import",
+    "emu_launch_count", "emu_host_launch_count", "emu_prof_enable", "emu_prof_read", "emu_prof_timeline", "emu_trace_enable", "emu_trace_read", "emu_potrf_task_list", "emu_test_wait_hook", "emu_test_sweep_hook", "emu_schedule", "emu_schedule_info", "emu_fp64_arithmetic", "emu_measure_alu_peaks", "emu_cov_build", "emu_mat_import",
     "emu_mat_import_host", "emu_cov_from_residuals", "emu_var_recursion", "emu_isht", "emu_sht", "emu_emulate_grid", "emu_cov_build_classfmt",
     "emu_backward_error_est", "emu_mat_clone", "emu_mat_export", "emu_mat_tile_info", "emu_mat_shape",
     "emu_mat_free", "emu_potrf_mp", "emu_sample", "emu_sample_host", "emu_potrs", "emu_solve_refine",
@@ -109,6 +109,7 @@ def load() -> ctypes.CDLL:
     L.emu_test_wait_hook.argtypes = [vp, ctypes.c_longlong, i]
     L.emu_test_sweep_hook.argtypes = [vp, ctypes.c_longlong, i]
     L.emu_schedule.argtypes = [vp, i, i]
+    L.emu_fp64_arithmetic.argtypes = [vp, i]
     L.emu_measure_alu_peaks.argtypes = [vp, dpp, dpp]
     L.emu_schedule_info.argtypes = [vp, ctypes.POINTER(i), ctypes.POINTER(i), ctypes.POINTER(i)]
     L.emu_prof_timeline.argtypes = [vp, vp, ctypes.c_size_t, ctypes.POINTER(ctypes.c_size_t)]
@@ -145,7 +146,7 @@ def load() -> ctypes.CDLL:
     for name in ("emu_create", "emu_destroy", "emu_set_stream", "emu_prof_enable", "emu_prof_read",
                  "emu_trace_enable", "emu_trace_read", "emu_potrf_task_list", "emu_prof_timeline",
                  "emu_test_wait_hook", "emu_test_sweep_hook",
-                 "emu_schedule", "emu_schedule_info", "emu_measure_alu_peaks",
+                 "emu_schedule", "emu_schedule_info", "emu_fp64_arithmetic", "emu_measure_alu_peaks",
                  "emu_mat_import_host", "emu_cov_build", "emu_mat_import", "emu_emulate_grid",
                  "emu_cov_build_classfmt", "emu_backward_error_est",
                  "emu_mat_clone", "emu_mat_export", "emu_mat_tile_info", "emu_mat_shape", "emu_mat_free",
@@ -234,6 +235,10 @@ class Context:
     def schedule(self, graphs: bool = True, tuning: bool = True):
         """Graph replay and reserved-SM tuning of the single-matrix mixed factor (both on by default)."""
         self._check(self.lib.emu_schedule(self.h, int(graphs), int(tuning)), "emu_schedule")
+
+    def fp64_arithmetic(self, on: bool = True):
+        """Plain FP64 factor, its draws and the transforms in FP64 arithmetic instead of digit products (off by default)."""
+        self._check(self.lib.emu_fp64_arithmetic(self.h, int(on)), "emu_fp64_arithmetic")
 
     def schedule_info(self):
         """(choices timed, SMs left free, SMs left free near FP64-class panel work) of the tuner."""

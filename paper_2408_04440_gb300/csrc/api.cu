@@ -230,6 +230,12 @@ emu_status emu_schedule_info(emu_ctx *ctx, int *tried, int *reserved, int *reser
   return EMU_OK;
 }
 
+emu_status emu_fp64_arithmetic(emu_ctx *ctx, int on) {
+  if (!ctx) return EMU_EINVAL;
+  ctx->fp64_pipe = on != 0;
+  return EMU_OK;
+}
+
 emu_status emu_test_wait_hook(emu_ctx *ctx, long long wait_cycles, int withhold_index) {
   if (!ctx) return EMU_EINVAL;
   EMU_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
@@ -615,7 +621,8 @@ static emu_status collect_status(emu_ctx *ctx, int *pivot) {
 }
 
 // Plain FP64 right-looking tile Cholesky on the FP64 pipe, for the tile sizes
-// the digit form does not take: POTRF(k), TRSM(:,k), SYRK/GEMM of the trailing
+// the digit form does not take, where its workspace does not fit, and by choice
+// (emu_fp64_arithmetic): POTRF(k), TRSM(:,k), SYRK/GEMM of the trailing
 // tiles, k = 0 .. NT-1.
 static emu_status factor64(emu_ctx *ctx, emu_mat *A) {
   for (int k = 0; k < A->nt; k++) {
@@ -644,7 +651,7 @@ extern "C" emu_status emu_potrf_mp(emu_ctx *ctx, emu_mat *A, const emu_mp_opts *
   } else if (mixed) {
     s = factor_mixed(ctx, A, o);
   } else {
-    s = factor64_digits_supports(A) ? factor64_digits(ctx, A) : EMU_ENOMEM;
+    s = !ctx->fp64_pipe && factor64_digits_supports(A) ? factor64_digits(ctx, A) : EMU_ENOMEM;
     if (s == EMU_ENOMEM) s = factor64(ctx, A);
   }
   if (s != EMU_OK) return s;
@@ -696,7 +703,8 @@ extern "C" emu_status emu_sample(emu_ctx *ctx, const emu_mat *L, int nsamples, u
     if (L->cs)
       s = classfmt_sample(ctx, L, Z, npad, nsamples, dY, ldy);
     else if (L->state == MAT_FACTOR64) {
-      s = factor64_digits_supports(L) ? sample64_digits(ctx, L, Z, npad, nsamples, dY, ldy) : EMU_ENOMEM;
+      s = !ctx->fp64_pipe && factor64_digits_supports(L) ? sample64_digits(ctx, L, Z, npad, nsamples, dY, ldy)
+                                                         : EMU_ENOMEM;
       if (s == EMU_ENOMEM) s = launch_trmm64(ctx, L, Z, npad, nsamples, dY, ldy);
     }
     else

@@ -103,6 +103,9 @@ struct emu_ctx {
   void *batch = nullptr;
   // single-matrix mixed factor (mixed.cu): captured graph, tuning table
   void *mixed = nullptr;
+  // emu_fp64_arithmetic: no digit products in the plain FP64 factor, its draws
+  // and the transforms
+  bool fp64_pipe = false;
   // test hook of the triangular sweeps: wait bound in cycles (0: default) and
   // the slab that is never published (-1: none)
   long long sweep_wait = 0;

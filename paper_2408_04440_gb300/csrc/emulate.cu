@@ -406,10 +406,13 @@ __global__ void __launch_bounds__(128) k_emulate_grid(const double *Zs, long G, 
 // (inverse / forward, us): L = 24, 100 steps (2.5e7, 3.7e7 flops) 111 against
 // 115 / 194 against 203, 30 steps 107 against 93 / 192 against 140; L = 48, one
 // step 116 against 133 / 217 against 334.
-static bool by_digits(int L, double flops) { return L >= 40 || flops >= 3e7; }
+static bool by_digits(const emu_ctx *ctx, int L, double flops) {
+  return !ctx->fp64_pipe && (L >= 40 || flops >= 3e7);
+}
 
 // The transforms' sums on the FP64 pipe: small transforms, operands with an
-// infinity or a NaN, and sizes whose digits do not fit the device.
+// infinity or a NaN, sizes whose digits do not fit the device, and by choice
+// (emu_fp64_arithmetic).
 static emu_status isht_direct(emu_ctx *ctx, const double *dF, int L, int T, long ldf, int ntheta, int nphi, double *dZ,
                               long ldz) {
   cudaStream_t s = ctx->stream;
@@ -496,7 +499,7 @@ emu_status emu_isht(emu_ctx *ctx, const double *dF, int L, int T, long ldf, int 
   EMU_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
   EMU_CUDA_TRY(ctx, status_clear(ctx));
   const double flops = 2.0 * (double)L * L * ntheta * T + 4.0 * (double)L * ntheta * nphi * T;
-  if (by_digits(L, flops)) {
+  if (by_digits(ctx, L, flops)) {
     ProfScope ps(ctx, PROF_SOLVE, flops, 0.0);
     const emu_status s = isht_digits(ctx, dF, L, T, ldf, ntheta, nphi, dZ, ldz);
     if (s != EMU_ENOMEM && s != EMU_ESTATE) return s;
@@ -515,7 +518,7 @@ emu_status emu_sht(emu_ctx *ctx, const double *dZ, int ntheta, int nphi, int T, 
   EMU_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
   EMU_CUDA_TRY(ctx, status_clear(ctx));
   const double flops = 4.0 * (double)L * ntheta * nphi * T + 4.0 * (double)L * Q * ntheta * T;
-  if (by_digits(L, flops)) {
+  if (by_digits(ctx, L, flops)) {
     ProfScope ps(ctx, PROF_SOLVE, flops, 0.0);
     const emu_status s = sht_digits(ctx, dZ, ntheta, nphi, T, ldz, L, dF, ldf);
     if (s != EMU_ENOMEM && s != EMU_ESTATE) return s;
