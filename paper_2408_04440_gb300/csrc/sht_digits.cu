@@ -346,9 +346,7 @@ emu_status sht_passes(emu_ctx *ctx, const double *dZ, int ntheta, int nphi, int 
          *cs = D(9);
   uint16_t *ld = U(10), *wd = U(11), *gd = U(12), *zd = U(13), *td = U(14), *rd = U(15);
   int *le = I(16), *we = I(17), *ge = I(18), *ze = I(19), *te = I(20), *re = I(21), *flag = I(22);
-  CUtensorMap ml, mw, mg, mz, mt, mr;
-  TRY(gemm64::make_map(ctx, &ml, ld, Ki, (uint64_t)NS * np, gemm64::BM));
-  TRY(gemm64::make_map(ctx, &mw, wd, Ki, (uint64_t)2 * NS * wpad, gemm64::BN));
+  CUtensorMap mg, mz, mt, mr;
   TRY(gemm64::make_map(ctx, &mg, gd, Ki, (uint64_t)NS * np, gemm64::BN));
   TRY(gemm64::make_map(ctx, &mz, zd, Kj, (uint64_t)NS * Rp, gemm64::BM));
   TRY(gemm64::make_map(ctx, &mt, td, Kj, (uint64_t)NS * nq, gemm64::BN));
