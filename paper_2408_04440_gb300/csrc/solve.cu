@@ -36,9 +36,11 @@ constexpr int LDD = 66;   // FP64 columns
 // default wait bound in SM clock cycles (about 2 s at 2 GHz)
 constexpr long long kSweepWaitCycles = 4000000000ll;
 // Published values of the groups of one launch: 16 bytes per FP32 entry of X in
-// both sweeps, 32 per FP64 one.  64 MB of them are 2000 slabs, several times the
-// CTAs that are resident; one group takes more from n = 130000 on.
-constexpr size_t kSweepWorkspace = (size_t)64 << 20;
+// both sweeps, 32 per FP64 one, up to this much (n = 65536 with 2000 right-hand
+// sides).  Every further launch is another ramp and tail of n / 64 slabs: with
+// 64 MB the 1000 right-hand sides of n = 16384 ran in five launches, 66.7 ms
+// instead of 56.4.
+constexpr size_t kSweepWorkspace = (size_t)2 << 30;
 
 __device__ inline bool failed(const int *st) { return *((volatile const int *)st) != DEV_OK; }
 
