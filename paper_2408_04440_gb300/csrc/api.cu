@@ -126,7 +126,7 @@ emu_status emu_create(emu_ctx **out, int device, void *stream) {
   ctx->sm_count = p.multiProcessorCount;
   cudaError_t e = cudaSetDevice(device);
   if (e == cudaSuccess) e = cudaMalloc(&ctx->d_status, ST_WORDS * sizeof(int));
-  if (e == cudaSuccess) e = cudaMallocHost(&ctx->h_status, (ST_WORDS + 1) * sizeof(int));
+  if (e == cudaSuccess) e = cudaMallocHost(&ctx->h_status, ST_WORDS * sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(ctx->d_status, 0, ST_WORDS * sizeof(int));
   if (e == cudaSuccess) e = cudaEventCreate(&ctx->ev0);
   if (e == cudaSuccess) e = cudaEventCreate(&ctx->ev1);

@@ -31,10 +31,11 @@ __host__ __device__ inline void tile_coords(long t, int NT, int *i, int *j) {
 inline long tile_count(int NT) { return (long)NT * (NT + 1) / 2; }
 
 // Device status word written by kernels and read back at sync points.  Calls
-// clear the words before ST_LATE when they begin.  ST_LATE stays: it records
+// clear the words before ST_LATE when they begin.  ST_FLAG is a call's own (the
+// transforms: an operand is not finite).  ST_LATE stays: it records
 // that a wait ran out, also in a call that returns before its device work ends
 // (emu_potrs, emu_sample), until a call that reads the status reports it.
-enum { ST_CODE = 0, ST_PIVOT = 1, ST_AUX = 2, ST_LATE = 3, ST_WORDS = 4 };
+enum { ST_CODE = 0, ST_PIVOT = 1, ST_AUX = 2, ST_FLAG = 3, ST_LATE = 4, ST_WORDS = 5 };
 enum { DEV_OK = 0, DEV_NOTPD = 1, DEV_TIMEOUT = 2 };
 __device__ inline void status_timeout(int *st, int aux) {
   if (atomicCAS(&st[ST_CODE], DEV_OK, DEV_TIMEOUT) == DEV_OK) st[ST_AUX] = aux;
@@ -64,7 +65,7 @@ struct emu_ctx {
   cudaStream_t stream = nullptr;
   int sm_count = 0;
   int *d_status = nullptr;    // ST_WORDS ints
-  int *h_status = nullptr;    // pinned mirror, and one more word for a call's own flag
+  int *h_status = nullptr;    // pinned mirror
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   uint64_t launches = 0;       // kernels of this library, graph nodes included
   uint64_t host_launches = 0;  // launch calls the host made (a graph replay counts once)

@@ -114,9 +114,10 @@ __global__ void k_symm_finish(const double *__restrict__ part, int nz, int P, co
   }
 }
 
-// Column sums of squares of R, X and B (one CTA per column, fixed order).
+// Column sums of squares of R, X and B (one CTA per column, fixed order), and
+// after them whether a wait ran out in the sweeps so far.
 __global__ void k_col_norms(const double *__restrict__ R, const double *__restrict__ X,
-                            const double *__restrict__ Bm, long n, long ld, double *__restrict__ out) {
+                            const double *__restrict__ Bm, long n, long ld, double *__restrict__ out, const int *st) {
   int c = blockIdx.x;
   double sr = 0, sx = 0, sb = 0;
   for (long r = threadIdx.x; r < n; r += blockDim.x) {
@@ -148,6 +149,7 @@ __global__ void k_col_norms(const double *__restrict__ R, const double *__restri
     out[3 * c] = a;
     out[3 * c + 1] = b;
     out[3 * c + 2] = d;
+    if (c == 0) out[3 * gridDim.x] = st[ST_CODE] == DEV_TIMEOUT || st[ST_LATE] ? 1.0 : 0.0;
   }
 }
 
@@ -188,9 +190,9 @@ emu_status refine_solve(emu_ctx *ctx, const emu_mat *L, const emu_mat *S, const 
   double *buf = nullptr, *norms = nullptr;
   const ResidualSplit sh = residual_split(ctx->sm_count, S->nt, S->nb, nrhs);
   EMU_CUDA_TRY(ctx, cudaMallocAsync(&buf, (4 * blk + sh.partial(npad)) * sizeof(double), ctx->stream));
-  EMU_CUDA_TRY(ctx, cudaMallocAsync(&norms, 3 * nrhs * sizeof(double), ctx->stream));
+  EMU_CUDA_TRY(ctx, cudaMallocAsync(&norms, (3 * (size_t)nrhs + 1) * sizeof(double), ctx->stream));
   double *Bp = buf, *X = buf + blk, *R = buf + 2 * blk, *D = buf + 3 * blk;
-  std::vector<double> hn(3 * nrhs);
+  std::vector<double> hn(3 * (size_t)nrhs + 1);
   double frobS = 0.0;
   emu_status s = EMU_OK;
   int it = 0;
@@ -210,16 +212,19 @@ emu_status refine_solve(emu_ctx *ctx, const emu_mat *L, const emu_mat *S, const 
   }
   while (s == EMU_OK) {
     if ((s = symm_residual(ctx, S, X, Bp, R, buf + 4 * blk, nrhs)) != EMU_OK) break;
-    k_col_norms<<<nrhs, 256, 0, ctx->stream>>>(R, X, Bp, npad, npad, norms);
+    k_col_norms<<<nrhs, 256, 0, ctx->stream>>>(R, X, Bp, npad, npad, norms, ctx->d_status);
     ctx->launches++;
     e = cudaGetLastError();
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(hn.data(), norms, 3 * nrhs * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(ctx->h_status, ctx->d_status, ST_WORDS * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
+      e = cudaMemcpyAsync(hn.data(), norms, hn.size() * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-    // a sweep that gave up has left X or its correction half solved
-    s = e == cudaSuccess ? status_timed_out(ctx) : emu_cuda_fail(ctx, e, "refine residual");
+    if (e == cudaSuccess && hn.back() != 0.0) {
+      // a sweep that gave up has left X or its correction half solved
+      e = cudaMemcpyAsync(ctx->h_status, ctx->d_status, ST_WORDS * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+      if (e == cudaSuccess) s = status_timed_out(ctx);
+    }
+    if (e != cudaSuccess) s = emu_cuda_fail(ctx, e, "refine residual");
     if (s != EMU_OK) break;
     eta = 0.0;
     for (int c = 0; c < nrhs; c++) {

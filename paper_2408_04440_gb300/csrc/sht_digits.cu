@@ -292,13 +292,12 @@ emu_status isht_passes(emu_ctx *ctx, const double *dF, int L, int T, long ldf, i
   auto I = [&](int k) { return reinterpret_cast<int *>(b + o[k]); };
   double *ca = D(0), *cr = D(1), *cq = D(2), *lam = D(3), *ab = D(4);
   uint16_t *ld = U(5), *fd = U(6), *ad = U(7), *td = U(8);
-  int *le = I(9), *fe = I(10), *ae = I(11), *te = I(12), *flag = I(13);
+  int *le = I(9), *fe = I(10), *ae = I(11), *te = I(12), *flag = ctx->d_status + ST_FLAG;
   CUtensorMap ml, mf, ma, mt;
   TRY(gemm64::make_map(ctx, &ml, ld, ktot, (uint64_t)NS * cpad, gemm64::BN));
   TRY(gemm64::make_map(ctx, &mf, fd, ktot, (uint64_t)NS * rpad, gemm64::BM));
   TRY(gemm64::make_map(ctx, &ma, ad, Kq, (uint64_t)NS * Rp, gemm64::BM));
   TRY(gemm64::make_map(ctx, &mt, td, Kq, (uint64_t)NS * npj, gemm64::BN));
-  EMU_CUDA_TRY(ctx, cudaMemsetAsync(flag, 0, sizeof(int), st));
   k_leg_coef<<<dim3((L + 127) / 128, L), 128, 0, st>>>(L, ca, cr, cq);
   EMU_LAUNCHED(ctx);
   k_legendre_fast<<<dim3((ntheta + 31) / 32, L), 32, 0, st>>>(L, ntheta, 0, ca, cr, cq, lam);
@@ -345,13 +344,12 @@ emu_status sht_passes(emu_ctx *ctx, const double *dZ, int ntheta, int nphi, int 
   double *ca = D(0), *cr = D(1), *cq = D(2), *lam = D(3), *cm = D(4), *ir = D(5), *P = D(6), *W = D(7), *G = D(8),
          *cs = D(9);
   uint16_t *ld = U(10), *wd = U(11), *gd = U(12), *zd = U(13), *td = U(14), *rd = U(15);
-  int *le = I(16), *we = I(17), *ge = I(18), *ze = I(19), *te = I(20), *re = I(21), *flag = I(22);
+  int *le = I(16), *we = I(17), *ge = I(18), *ze = I(19), *te = I(20), *re = I(21), *flag = ctx->d_status + ST_FLAG;
   CUtensorMap mg, mz, mt, mr;
   TRY(gemm64::make_map(ctx, &mg, gd, Ki, (uint64_t)NS * np, gemm64::BN));
   TRY(gemm64::make_map(ctx, &mz, zd, Kj, (uint64_t)NS * Rp, gemm64::BM));
   TRY(gemm64::make_map(ctx, &mt, td, Kj, (uint64_t)NS * nq, gemm64::BN));
   TRY(gemm64::make_map(ctx, &mr, rd, Ki, (uint64_t)NS * L * rpad, gemm64::BM));
-  EMU_CUDA_TRY(ctx, cudaMemsetAsync(flag, 0, sizeof(int), st));
   k_leg_coef<<<dim3((L + 127) / 128, L), 128, 0, st>>>(L, ca, cr, cq);
   EMU_LAUNCHED(ctx);
   k_legendre_fast<<<dim3((ntheta + 31) / 32, L), 32, 0, st>>>(L, ntheta, 1, ca, cr, cq, lam);
@@ -415,19 +413,16 @@ emu_status sht_passes(emu_ctx *ctx, const double *dZ, int ntheta, int nphi, int 
 }
 
 // Waits for the transform: EMU_ESTATE when an operand held an infinity or a NaN.
-emu_status finish(emu_ctx *ctx, char *blob, const int *flag, emu_status s) {
+emu_status finish(emu_ctx *ctx, char *blob, emu_status s) {
   cudaError_t e = cudaSuccess;
-  if (s == EMU_OK) {
+  if (s == EMU_OK)
     e = cudaMemcpyAsync(ctx->h_status, ctx->d_status, ST_WORDS * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(ctx->h_status + ST_WORDS, flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
-  }
   cudaFreeAsync(blob, ctx->stream);
   if (s != EMU_OK) return s;
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) return emu_cuda_fail(ctx, e, "transform");
   s = status_timed_out(ctx);
-  return s != EMU_OK ? s : ctx->h_status[ST_WORDS] ? EMU_ESTATE : EMU_OK;
+  return s != EMU_OK ? s : ctx->h_status[ST_FLAG] ? EMU_ESTATE : EMU_OK;
 }
 
 }  // namespace
@@ -458,11 +453,10 @@ emu_status isht_digits(emu_ctx *ctx, const double *dF, int L, int T, long ldf, i
   o[10] = p.add(L * rpad * 4);
   o[11] = p.add(Rp * 4);
   o[12] = p.add(npj * 4);
-  o[13] = p.add(4);
   char *b = nullptr;
   TRY(alloc(ctx, &b, p.off));
   const emu_status s = isht_passes(ctx, dF, L, T, ldf, ntheta, nphi, dZ, ldz, b, Tc, o);
-  return finish(ctx, b, reinterpret_cast<int *>(b + o[13]), s);
+  return finish(ctx, b, s);
 }
 
 emu_status sht_digits(emu_ctx *ctx, const double *dZ, int ntheta, int nphi, int T, long ldz, int L, double *dF,
@@ -495,9 +489,8 @@ emu_status sht_digits(emu_ctx *ctx, const double *dZ, int ntheta, int nphi, int 
   o[19] = p.add(Rp * 4);
   o[20] = p.add(nq * 4);
   o[21] = p.add(L * rpad * 4);
-  o[22] = p.add(4);
   char *b = nullptr;
   TRY(alloc(ctx, &b, p.off));
   const emu_status s = sht_passes(ctx, dZ, ntheta, nphi, T, ldz, L, dF, ldf, b, Tc, o);
-  return finish(ctx, b, reinterpret_cast<int *>(b + o[22]), s);
+  return finish(ctx, b, s);
 }
