@@ -1123,7 +1123,8 @@ def run_fp64_L400(a):
         A = E.emu_cov_build(ctx, L, beta, nb)
         clocks.start()
         info = E.emu_potrf_mp(ctx, A)
-        out["fp64_pipe"] = {"factor_s": round(info.ms / 1e3, 2), "tflops": round(flops / (info.ms * 1e-3) / 1e12, 4),
+        out["fp64_plain"] = {"form": "digit products (FP64 arithmetic by choice: emu_fp64_arithmetic)",
+                             "factor_s": round(info.ms / 1e3, 2), "tflops": round(flops / (info.ms * 1e-3) / 1e12, 4),
                             "backward_error_est": E.emu_backward_error_est(ctx, A, L, beta, nprobes=4, seed=5),
                             "clocks": clocks.stop()}
         A.free()

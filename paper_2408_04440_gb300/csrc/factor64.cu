@@ -7,6 +7,13 @@
 // n u sqrt(S_ii S_jj) of the factor formed in FP64 arithmetic, with 2^-56 in
 // place of u.
 //
+// Entries of L far below that scale are less accurate relative to themselves
+// than FP64 arithmetic makes them: against its own bound, n u (|L| |L|^T)_ij,
+// the error reaches 1500 times that on the synthetic covariance (n = 1024, beta =
+// 3; the largest relative error of an entry 1e-9 at n = 400) and far more on a
+// matrix whose off-diagonal entries span fourteen decades, at the same norm of
+// the error.  emu_fp64_arithmetic keeps a context on FP64 sums.
+//
 // Why: the FP64 pipe does 1.2 TFLOP/s, the 36 digit products of a K step run
 // at 45 TFLOP/s of FP64 work.  What stays on the FP64 pipe is the diagonal
 // POTRF and the 128-column block solves of the panel.
@@ -84,8 +91,17 @@ emu_status plan_make(emu_ctx *ctx, const emu_mat *A, Plan *P) {
 
 // SMs the bulk update leaves to the panel work: a bulk CTA fills its SM's
 // registers and shared memory, and the block solves are bound by the FP64
-// pipes of the SMs they find (n = 10000, nb = 512: 24.8 ms with 16, 24.4 with
-// 32, 24.1 with 48, 24.2 with 64).
+// pipes of the SMs they find.  Panel work grows as n nb, the update as n^2, so
+// the best count falls with n / nb.  Factor in ms with 16 / 32 / 48 / 64:
+//   n =  1600, nb =  128    1.65 / 1.65 / 1.64 / 1.63
+//   n =  4096, nb =  256    4.56 / 4.58 / 4.57 / 4.57
+//   n = 10000, nb =  512    21.7 / 21.4 / 21.3 / 21.3
+//   n = 16384, nb =  512    62.9 / 61.4 / 60.9 / 62.7
+//   n = 16384, nb = 1024    66.4 / 66.4 / 66.3 / 65.7
+//   n = 40000, nb = 1024     660 /  651 /  682 /  773
+//   n = 65536, nb = 1024    2380 / 2480 / 2780 / 3220
+// 48 is the best up to n = 20000 or so and loses 5 % at 40000 and 17 % at 65536,
+// where a count that follows the ratio of the two kinds of work would pay.
 constexpr int kReserved = 48;
 
 emu_status factor_launches(emu_ctx *ctx, emu_mat *A, Plan *P) {

@@ -2,7 +2,7 @@
 // FP64-class tiles of the mixed-precision factor (see gemm_f64.h for the
 // digit scheme and why every tensor-core sum is exact).
 //
-// Warp roles (192 threads, one CTA per SM, persistent over the item list):
+// Warp roles (640 threads, one CTA per SM, persistent over the item list):
 //   warp 0      TMA producer: per K stage the NS digit planes of the A block
 //               (128 x 32) and of the B block (64 x 32), 96 KB.
 //   warp 1      TMEM allocator + MMA issuer: per 16-deep K step the 36 digit
