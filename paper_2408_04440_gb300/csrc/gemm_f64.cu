@@ -757,10 +757,14 @@ __global__ void __maxnreg__(96)
 #pragma unroll
           for (int x = 0; x < 8; x++) {
             const int cx = col0 + x0 + x;
-            double v = fixed_scaled(hi[x0 + x], lo[x0 + x], ea + exp_of(b_exp, (long)item.b_sc + cx));
+            // columns past the last hold whatever the arena held: exponents there
+            // can send fixed_scaled to its slow form (a third of the columns of
+            // 129 rings, 40 of 135 us of the synthesis' products)
+            if (!kWhole && cx >= item.cols_valid) continue;
+            const double v = fixed_scaled(hi[x0 + x], lo[x0 + x], ea + exp_of(b_exp, (long)item.b_sc + cx));
             if (MODE == TC64_SUB)
               __stcg(o + (long)cx * ldo, cv[x] - v);
-            else if (kWhole || cx < item.cols_valid) {
+            else {
               if constexpr (SRC == SRC_ANA) {
                 // order +-m, degree l = m + column; the sine sums of order 0 have no coefficient
                 const long l = item.m + item.col0 + cx;
